@@ -588,7 +588,7 @@ def run(args):
     m32 = measure(params, args.steps, args.warmup)
     clk = clocks.stop()
     value, ms_max, out = m32["value"], m32["ms"], m32["out"]
-    digest = src_digest("search.cu", "common.cuh", "warp_ops.cuh", "internal.h")
+    digest = src_digest("search.cu", "search_kernel.cuh", "common.cuh", "warp_ops.cuh", "internal.h")
     traffic, capture = traffic_for(digest, name, params)
     roofline = {"bound": "hbm", "achieved": m32["achieved"], "peak": hbm, "unit": "GB/s",
                 "frac": m32["achieved"] / hbm, "traffic": traffic,

@@ -96,10 +96,11 @@ typedef struct {
   int max_expansions;  /* expansions per layer before UNIFY_Q_LIMIT, default 100000 */
   int warps_per_block; /* search warps per CTA (one query or scan item each), 1..4, default 4 */
   int scan_rows;       /* pre-filter rows per scan work item, default 8192 */
-  int reg_budget;      /* registers per thread of the search kernel: 128 (16 warps per SM),
-                          80 (24 warps) or 64 (32 warps, smaller distance groups); default 128.
-                          More resident warps hide more memory latency when shared memory
-                          (cand_cap, visited_cap, ef) also fits. */
+  int reg_budget;      /* build of the search kernel for rows of up to 128 elements: 128 (128 registers
+                          per thread, 16 warps per SM), 80 (96 registers, 20 warps) or 64 (80
+                          registers, 24 warps; the smaller builds hold fewer rows in flight per
+                          warp); default 128. More resident warps hide more memory latency when
+                          shared memory (cand_cap, visited_cap, ef) also fits. */
   int tc_scan;         /* 1: Strategy A queries are scanned on the tensor cores (tcgen05 MMA
                           over TMA-staged row tiles shared by 128 queries; bf16 operands for
                           UNIFY_BF16 storage, tf32 for UNIFY_FP32, E4M3 for UNIFY_FP8E4M3; the

@@ -81,27 +81,29 @@ struct BuildArgs {
 };
 
 struct BuildWarp {
-  uint64_t* E;
-  uint8_t* Ef;
-  int32_t* vis;
-  int* R;
-  int* clist;
+  float4* q;   // the inserted node's row
+  float4* xr;  // pruning: the candidate's row
+  uint64_t* SK;
   uint64_t* kept;
+  int* clist;
+  int32_t* vis;
+  uint64_t* E;
 };
 
-__host__ __device__ inline size_t build_warp_bytes(int ecap) {
-  size_t b = (size_t)ecap * 8 + (size_t)((ecap + 15) & ~15) + ((size_t)4 << kBuildVisLog2) + 32 * 4 * 2 + 32 * 8;
+__host__ __device__ inline size_t build_warp_bytes(int ecap, int dp4) {
+  const size_t b = (size_t)dp4 * 32 + 32 * 8 * 2 + 32 * 4 + ((size_t)4 << kBuildVisLog2) + (size_t)ecap * 8;
   return (b + 15) & ~(size_t)15;
 }
 
-__device__ __forceinline__ BuildWarp build_carve(unsigned char* base, int ecap) {
+__device__ __forceinline__ BuildWarp build_carve(unsigned char* base, int dp4) {
   BuildWarp w;
-  w.E = reinterpret_cast<uint64_t*>(base);
-  w.Ef = reinterpret_cast<uint8_t*>(w.E + ecap);
-  w.vis = reinterpret_cast<int32_t*>(w.Ef + ((ecap + 15) & ~15));
-  w.R = reinterpret_cast<int*>(w.vis + (1 << kBuildVisLog2));
-  w.clist = w.R + 32;
-  w.kept = reinterpret_cast<uint64_t*>(w.clist + 32);
+  w.q = reinterpret_cast<float4*>(base);
+  w.xr = w.q + dp4;
+  w.SK = reinterpret_cast<uint64_t*>(w.xr + dp4);
+  w.kept = w.SK + 32;
+  w.clist = reinterpret_cast<int*>(w.kept + 32);
+  w.vis = w.clist + 32;
+  w.E = reinterpret_cast<uint64_t*>(w.vis + (1 << kBuildVisLog2));
   return w;
 }
 
@@ -109,7 +111,7 @@ __device__ __forceinline__ uint32_t build_hash(int id) {
   return ((uint32_t)id * 0x9E3779B1u) >> (32 - kBuildVisLog2);
 }
 
-// Row id of X into the lane layout (chunks lane, lane + 32, ...).
+// Row id of X into this lane's registers (chunks lane, lane + 32, ...).
 template <int CH>
 __device__ __forceinline__ void load_row(float4 (&x)[CH], const float* X, int dp4, int64_t id) {
   const int lane = lane_id();
@@ -121,85 +123,127 @@ __device__ __forceinline__ void load_row(float4 (&x)[CH], const float* X, int dp
   }
 }
 
+// The row in x to shared memory, for the whole warp.
+template <int CH>
+__device__ __forceinline__ void share_row(float4* dst, const float4 (&x)[CH], int dp4) {
+  const int lane = lane_id();
+  __syncwarp();
+#pragma unroll
+  for (int t = 0; t < CH; ++t) {
+    const int c = lane + 32 * t;
+    if (c < dp4) dst[c] = x[t];
+  }
+  __syncwarp();
+}
+
+// Keys of E: (distance bits) << 32 | id << 1 | expanded (n < 2^30).
+__device__ __forceinline__ uint64_t edge_key(float d, int id) {
+  return ((uint64_t)__float_as_uint(d) << 32) | ((uint32_t)id << 1);
+}
+__device__ __forceinline__ int edge_id(uint64_t k) { return (int)((uint32_t)k >> 1); }
+
 // ANNSearch (Algorithm 1) from ep_key on layer l over the chunks j, capacity ef.
 // Returns |E|; E[0, |E|) ascending.
 template <int CH, int G>
-__device__ int build_search(const BuildArgs& a, const BuildWarp& w, const float4 (&q)[CH], int l, int j, int ef,
-                            uint64_t ep_key) {
+__device__ int build_search(const BuildArgs& a, const BuildWarp& w, int l, int j, int ef, uint64_t ep_key) {
   const int lane = lane_id();
-  for (int t = lane; t < (1 << kBuildVisLog2); t += 32) w.vis[t] = -1;
+  for (int t = lane; t < (1 << kBuildVisLog2) / 4; t += 32)
+    reinterpret_cast<int4*>(w.vis)[t] = make_int4(-1, -1, -1, -1);
   __syncwarp();
-  const int ep = key_id(ep_key);
+  const int ep = edge_id(ep_key);
   if (lane == 0) {
     w.E[0] = ep_key;
-    w.Ef[0] = 0;
     w.vis[build_hash(ep)] = ep;
   }
   __syncwarp();
   int nE = 1, cursor = 0;
   long long nexp = 0;
+  int ahead = -1, acid = -1;  // object whose neighbours lane by lane are in acid
   for (;;) {
-    // the nearest unexpanded candidate
+    // the nearest unexpanded candidate, and the one after it among the next 31 entries
+    int o = -1, o2 = -1;
     while (cursor < nE) {
       const int jj = cursor + lane;
-      const unsigned bal = __ballot_sync(kFull, jj < nE && w.Ef[jj] == 0);
+      const uint32_t lo = jj < nE ? (uint32_t)w.E[jj] : 1u;
+      const unsigned bal = __ballot_sync(kFull, (lo & 1u) == 0u);
       if (bal) {
-        cursor += __ffs(bal) - 1;
+        const int at = __ffs(bal) - 1;
+        const unsigned rest = bal & (bal - 1);
+        o = (int)(__shfl_sync(kFull, lo, at) >> 1);
+        if (rest) o2 = (int)(__shfl_sync(kFull, lo, __ffs(rest) - 1) >> 1);
+        if (lane == at) *reinterpret_cast<uint32_t*>(w.E + jj) = lo | 1u;
+        cursor += at;
         break;
       }
       cursor += 32;
     }
-    if (cursor >= nE) break;
+    if (o < 0) break;
     if (++nexp > kBuildMaxExpansions) {
       if (lane == 0) atomicExch(a.err, 1);
       break;
     }
-    const int o = key_id(w.E[cursor]);
     __syncwarp();
-    if (lane == 0) w.Ef[cursor] = 1;
-    __syncwarp();
-    const int64_t row = a.row0[o] + l;
-    const int c = a.cnt[row * a.S + j];
-    int cid = lane < c ? __ldg(a.adj + (row * a.S + j) * a.M + lane) : -1;
+    // slots past the count hold -1
+    int cid = acid;
+    if (ahead != o) {
+      const int64_t row = a.row0[o] + l;
+      cid = lane < a.M ? __ldg(a.adj + (row * a.S + j) * a.M + lane) : -1;
+    }
+    // the next candidate's neighbours, in flight behind this expansion's rows
+    ahead = o2;
+    const int64_t row2 = o2 >= 0 ? __ldg(a.row0 + o2) + l : 0;
     if (cid >= 0) {
       const uint32_t h = build_hash(cid);
       if (w.vis[h] == cid) cid = -1;
       else w.vis[h] = cid;
     }
     __syncwarp();
-    const float dist = batch_dist<StoreF32, CH, G>(q, cid, reinterpret_cast<const unsigned char*>(a.X), a.dp4 * 16,
-                                                   nullptr, a.dp4, w.clist);
-    const uint64_t key = cid >= 0 ? make_key(dist, cid) : kKeyMax;
-    const uint64_t thr = nE >= ef ? w.E[ef - 1] : kKeyMax;
-    bool keep = cid >= 0 && key < thr;
+    const unsigned vm = __ballot_sync(kFull, cid >= 0);
+    const int nc = __popc(vm);
+    if (cid >= 0) w.clist[__popc(vm & lanemask_lt())] = cid;
+    __syncwarp();
+    acid = o2 >= 0 && lane < a.M ? __ldg(a.adj + (row2 * a.S + j) * a.M + lane) : -1;
+    if (nc == 0) continue;
+    const int id = lane < nc ? w.clist[lane] : 0;
+    const float dist = group_dist<StoreF32, CH, G>(sa(w.q), sa(w.clist), nc, reinterpret_cast<const unsigned char*>(a.X),
+                                                   a.dp4 * 16, nullptr, a.dp4);
+    const uint64_t key = edge_key(dist, id);
+    const uint64_t thr = nE >= ef ? w.E[ef - 1] & ~1ull : kKeyMax;
+    bool keep = lane < nc && key < thr;
     // a visited object the filter forgot is still in E (or above the threshold)
-    if (keep && contains_u64(w.E, nE, key)) keep = false;
-    const unsigned kb = __ballot_sync(kFull, keep);
+    unsigned kb = __ballot_sync(kFull, keep);
     if (kb == 0) continue;
-    const uint64_t sk = warp_sort_asc(keep ? key : kKeyMax);
-    int r0;
-    bool dropped;
-    nE = warp_merge(w.E, w.Ef, nE, ef, sk, __popc(kb), w.R, &r0, &dropped);
+    const int rk = warp_rank(sa(w.E), nE, key, kb);
+    if (keep && rk < nE && (w.E[rk] ^ key) <= 1ull) keep = false;
+    kb = __ballot_sync(kFull, keep);
+    if (kb == 0) continue;
+    const int less = rank_among(key, kb, sa(w.SK));
+    nE = sorted_insert(sa(w.E), nE, ef, key, rk, less, kb);
+    const int r0 = (int)__reduce_min_sync(kFull, keep ? (unsigned)rk : 0x7fffffffu);
     if (r0 < cursor) cursor = r0;
   }
   __syncwarp();
   return nE;
 }
 
-// Pruning heuristic over E[0, nE): at most M kept keys in w.kept, ascending.
+// Pruning heuristic over E[0, nE): at most M kept keys in w.kept, ascending. The row of
+// the candidate after the current one is always on its way.
 template <int CH, int G>
 __device__ int build_prune(const BuildArgs& a, const BuildWarp& w, int nE) {
   const int lane = lane_id();
   int nk = 0;
+  float4 xr[CH];
+  load_row<CH>(xr, a.X, a.dp4, edge_id(w.E[0]));
   for (int i = 0; i < nE && nk < a.M; ++i) {
     const uint64_t r = w.E[i];
-    float4 xr[CH];
-    load_row<CH>(xr, a.X, a.dp4, key_id(r));
-    const int cid = lane < nk ? key_id(w.kept[lane]) : -1;
+    share_row<CH>(w.xr, xr, a.dp4);
+    if (i + 1 < nE) load_row<CH>(xr, a.X, a.dp4, edge_id(w.E[i + 1]));
+    if (lane < nk) w.clist[lane] = edge_id(w.kept[lane]);
+    __syncwarp();
     // distances from r to the kept objects, one per lane
-    const float dk = batch_dist<StoreF32, CH, G>(xr, cid, reinterpret_cast<const unsigned char*>(a.X), a.dp4 * 16,
-                                                 nullptr, a.dp4, w.clist);
-    const bool drop = __any_sync(kFull, cid >= 0 && key_dist(r) > dk);
+    const float dk = group_dist<StoreF32, CH, G>(sa(w.xr), sa(w.clist), nk, reinterpret_cast<const unsigned char*>(a.X),
+                                                 a.dp4 * 16, nullptr, a.dp4);
+    const bool drop = __any_sync(kFull, lane < nk && key_dist(r) > dk);
     if (!drop) {
       if (lane == 0) w.kept[nk] = r;
       ++nk;
@@ -210,10 +254,10 @@ __device__ int build_prune(const BuildArgs& a, const BuildWarp& w, int nE) {
 }
 
 template <int CH, int G>
-__global__ void __launch_bounds__(32 * kBuildWarps) build_kernel(BuildArgs a) {
+__global__ void __launch_bounds__(32 * kBuildWarps, 4) build_kernel(BuildArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = lane_id();
-  const BuildWarp w = build_carve(smem_raw + (size_t)warp * build_warp_bytes(a.ecap), a.ecap);
+  const BuildWarp w = build_carve(smem_raw + (size_t)warp * build_warp_bytes(a.ecap, a.dp4), a.dp4);
   const int64_t wid = (int64_t)blockIdx.x * kBuildWarps + warp;
   if (wid >= a.count * a.S) return;  // whole warps
   const int64_t t = wid / a.S;
@@ -226,26 +270,29 @@ __global__ void __launch_bounds__(32 * kBuildWarps) build_kernel(BuildArgs a) {
   const int ep0 = a.entry_seg[j];
   if (ep0 < 0) return;  // the segment holds no node yet
   const int L = a.top_seg[j];
-  float4 q[CH];
-  load_row<CH>(q, a.X, a.dp4, v);
-  const float d0 = batch_dist<StoreF32, CH, G>(q, lane == 0 ? ep0 : -1, reinterpret_cast<const unsigned char*>(a.X),
-                                               a.dp4 * 16, nullptr, a.dp4, w.clist);
-  uint64_t ep = make_key(__shfl_sync(kFull, d0, 0), ep0);
+  {
+    float4 q[CH];
+    load_row<CH>(q, a.X, a.dp4, v);
+    share_row<CH>(w.q, q, a.dp4);
+  }
+  const float d0 = batch_dist<StoreF32, CH, G>(sa(w.q), lane == 0 ? ep0 : -1, reinterpret_cast<const unsigned char*>(a.X),
+                                               a.dp4 * 16, nullptr, a.dp4, sa(w.clist));
+  uint64_t ep = edge_key(__shfl_sync(kFull, d0, 0), ep0);
   for (int l = L; l > lv; --l) {
-    build_search<CH, G>(a, w, q, l, j, 1, ep);
-    ep = w.E[0];
+    build_search<CH, G>(a, w, l, j, 1, ep);
+    ep = w.E[0] & ~1ull;
     __syncwarp();
   }
   for (int l = (lv < L ? lv : L); l >= 0; --l) {
-    const int nE = build_search<CH, G>(a, w, q, l, j, a.efc, ep);
+    const int nE = build_search<CH, G>(a, w, l, j, a.efc, ep);
     const int nk = build_prune<CH, G>(a, w, nE);
     const int64_t o = (rb + l) * a.S + j;
     for (int s = lane; s < nk; s += 32) {
-      a.out_ids[o * a.M + s] = key_id(w.kept[s]);
+      a.out_ids[o * a.M + s] = edge_id(w.kept[s]);
       a.out_dist[o * a.M + s] = key_dist(w.kept[s]);
     }
     if (lane == 0) a.out_cnt[o] = (uint8_t)nk;
-    ep = w.E[0];
+    ep = w.E[0] & ~1ull;
     __syncwarp();
   }
 }
@@ -300,10 +347,12 @@ struct RevArgs {
 // heuristic of Section 2.2 (candidates ascending; one is dropped when it is farther
 // from the owner than from a neighbour already kept).
 template <int CH, int G>
-__global__ void __launch_bounds__(32 * kBuildWarps) reverse_kernel(RevArgs a) {
+__global__ void __launch_bounds__(32 * kBuildWarps, 4) reverse_kernel(RevArgs a) {
   __shared__ uint64_t sK[kBuildWarps][kBuildMaxM + 1];
   __shared__ uint64_t sKept[kBuildWarps][kBuildMaxM];
   __shared__ int sList[kBuildWarps][32];
+  __shared__ float4 sRow[kBuildWarps][32 * CH];
+  __shared__ __align__(16) uint64_t sSK[kBuildWarps][32];
   const int warp = threadIdx.x >> 5, lane = lane_id();
   const int64_t g = (int64_t)blockIdx.x * kBuildWarps + warp;
   if (g >= a.ngroups) return;  // whole warps
@@ -312,8 +361,9 @@ __global__ void __launch_bounds__(32 * kBuildWarps) reverse_kernel(RevArgs a) {
   const int64_t ch = a.g_chunk[g];
   const int M = a.M;
   int c = a.cnt[ch];
-  uint64_t key = lane < c ? make_key(a.adjd[ch * M + lane], a.adj[ch * M + lane]) : kKeyMax;
-  K[lane] = warp_sort_asc(key);
+  const uint64_t key = lane < c ? make_key(a.adjd[ch * M + lane], a.adj[ch * M + lane]) : kKeyMax;
+  const int at = rank_plain(key, __ballot_sync(kFull, lane < c), sa(sSK[warp]));
+  if (lane < c) K[at] = key;
   __syncwarp();
   const int64_t e1 = a.g_start[g + 1];
   for (int64_t e = a.g_start[g]; e < e1; ++e) {
@@ -330,14 +380,18 @@ __global__ void __launch_bounds__(32 * kBuildWarps) reverse_kernel(RevArgs a) {
     ++c;
     if (c <= M) continue;
     int nk = 0;
+    float4 xr[CH];
+    load_row<CH>(xr, a.X, a.dp4, key_id(K[0]));
     for (int t = 0; t < c && nk < M; ++t) {
       const uint64_t r = K[t];
-      float4 xr[CH];
-      load_row<CH>(xr, a.X, a.dp4, key_id(r));
-      const int cid = lane < nk ? key_id(kept[lane]) : -1;
-      const float dk = batch_dist<StoreF32, CH, G>(xr, cid, reinterpret_cast<const unsigned char*>(a.X), a.dp4 * 16,
-                                                   nullptr, a.dp4, sList[warp]);
-      if (!__any_sync(kFull, cid >= 0 && key_dist(r) > dk)) {
+      share_row<CH>(sRow[warp], xr, a.dp4);
+      if (t + 1 < c) load_row<CH>(xr, a.X, a.dp4, key_id(K[t + 1]));
+      if (lane < nk) sList[warp][lane] = key_id(kept[lane]);
+      __syncwarp();
+      const float dk = group_dist<StoreF32, CH, G>(sa(sRow[warp]), sa(sList[warp]), nk,
+                                                   reinterpret_cast<const unsigned char*>(a.X), a.dp4 * 16, nullptr,
+                                                   a.dp4);
+      if (!__any_sync(kFull, lane < nk && key_dist(r) > dk)) {
         if (lane == 0) kept[nk] = r;
         ++nk;
         __syncwarp();
@@ -422,7 +476,7 @@ void build_free(BuildCtx* c) {
 
 template <int CH, int G>
 cudaError_t launch_build(const BuildArgs& a, cudaStream_t st) {
-  const size_t smem = (size_t)kBuildWarps * build_warp_bytes(a.ecap);
+  const size_t smem = (size_t)kBuildWarps * build_warp_bytes(a.ecap, a.dp4);
   cudaError_t e = cudaFuncSetAttribute(build_kernel<CH, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int64_t pairs = a.count * a.S;
@@ -528,10 +582,10 @@ int propose(BuildCtx* c, const unify_build_view_t* v, int32_t* out_ids, float* o
   a.out_cnt = c->o_cnt;
   a.err = c->err;
   const int ch = (a.dp4 + 31) / 32;
-  if (ch <= 1) e = launch_build<1, 16>(a, c->st);
+  if (ch <= 1) e = launch_build<1, 8>(a, c->st);
   else if (ch <= 2) e = launch_build<2, 8>(a, c->st);
-  else if (ch <= 4) e = launch_build<4, 4>(a, c->st);
-  else e = launch_build<8, 2>(a, c->st);
+  else if (ch <= 4) e = launch_build<4, 8>(a, c->st);
+  else e = launch_build<8, 8>(a, c->st);
   if (e != cudaSuccess) return bcuda_fail(e, "build assist: proposal kernel");
   int32_t herr = 0;
   e = cudaMemcpyAsync(out_ids, c->o_ids, rows * c->S * c->M * 4, cudaMemcpyDeviceToHost, c->st);
@@ -602,10 +656,10 @@ int apply(BuildCtx* c, const unify_build_view_t* v, const int64_t* g_chunk, cons
   a.r_v = c->r_v;
   a.r_d = c->r_d;
   const int chn = (a.dp4 + 31) / 32;
-  if (chn <= 1) e = launch_reverse<1, 16>(a, c->st);
+  if (chn <= 1) e = launch_reverse<1, 8>(a, c->st);
   else if (chn <= 2) e = launch_reverse<2, 8>(a, c->st);
-  else if (chn <= 4) e = launch_reverse<4, 4>(a, c->st);
-  else e = launch_reverse<8, 2>(a, c->st);
+  else if (chn <= 4) e = launch_reverse<4, 8>(a, c->st);
+  else e = launch_reverse<8, 8>(a, c->st);
   if (e != cudaSuccess) return bcuda_fail(e, "unify_build_apply: reverse-edge kernel");
   e = cudaStreamSynchronize(c->st);
   return e == cudaSuccess ? UNIFY_OK : bcuda_fail(e, "unify_build_apply");

@@ -24,175 +24,123 @@ __device__ __forceinline__ uint64_t make_key(float d, int32_t id) {
 __device__ __forceinline__ float key_dist(uint64_t k) { return __uint_as_float((uint32_t)(k >> 32)); }
 __device__ __forceinline__ int32_t key_id(uint64_t k) { return (int32_t)(uint32_t)(k & 0xffffffffu); }
 
-__device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
-__device__ __forceinline__ unsigned lanemask_lt() { return (1u << lane_id()) - 1u; }
-
-// Bitonic sort of one key per lane, ascending across lanes 0..31.
-__device__ __forceinline__ uint64_t warp_sort_asc(uint64_t x) {
-  const int lane = lane_id();
-#pragma unroll
-  for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      uint64_t y = __shfl_xor_sync(kFull, x, j);
-      bool up = (lane & k) == 0;
-      bool lower = (lane & j) == 0;
-      x = (lower == up) ? (x < y ? x : y) : (x < y ? y : x);
-    }
-  }
-  return x;
+// The lane, in a form that the compiler does not connect between calls: values derived
+// from it are recomputed where they are needed (an instruction or two) instead of being
+// kept in registers, or spilled, across a whole kernel.
+__device__ __forceinline__ int lane_id() {
+  int l = threadIdx.x & 31;
+  asm volatile("" : "+r"(l));
+  return l;
+}
+__device__ __forceinline__ unsigned lanemask_lt() {
+  unsigned m;
+  asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+  return m;
 }
 
-// The same network carrying a 32-bit payload with each key.
-__device__ __forceinline__ void warp_sort_asc_payload(uint64_t& x, uint32_t& f) {
-  const int lane = lane_id();
-#pragma unroll
-  for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      const uint64_t y = __shfl_xor_sync(kFull, x, j);
-      const uint32_t g = __shfl_xor_sync(kFull, f, j);
-      const bool up = (lane & k) == 0;
-      const bool lower = (lane & j) == 0;
-      const bool take = (lower == up) ? (y < x) : (x < y);
-      if (take) {
-        x = y;
-        f = g;
-      }
-    }
+// Shared memory by 32-bit address: plain ld.shared / st.shared whatever the compiler can
+// prove about a pointer, and one register per address. Volatile: they keep their order
+// among each other and with __syncwarp.
+using saddr = uint32_t;
+__device__ __forceinline__ saddr sa(const void* p) { return static_cast<saddr>(__cvta_generic_to_shared(p)); }
+__device__ __forceinline__ uint64_t lds64(saddr a) {
+  uint64_t v;
+  asm volatile("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t lds32(saddr a) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ ulonglong2 lds64x2(saddr a) {
+  ulonglong2 v;
+  asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ float4 lds_f4(saddr a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts64(saddr a, uint64_t v) { asm volatile("st.shared.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory"); }
+__device__ __forceinline__ void sts32(saddr a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+
+// Number of entries of the sorted array of n keys at a that are below x (per lane): a
+// binary search of a fixed number of steps (n is the same on every lane).
+__device__ __forceinline__ int lower_bound_u64(saddr a, int n, uint64_t x) {
+  int lo = 0;
+#pragma unroll 1
+  for (int step = n > 0 ? 1 << (31 - __clz(n)) : 0; step > 0; step >>= 1) {
+    const int i = lo + step;
+    if (i <= n && lds64(a + 8 * (i - 1)) < x) lo = i;
   }
+  return lo;
 }
 
-// The keys of the lanes in kb (a ballot; the other lanes hold kKeyMax), distinct,
-// sorted ascending into lanes 0 .. popc(kb) - 1 with their payloads; the other lanes
-// end with kKeyMax and payload 0. Up to four keys take their rank among the kept keys
-// by broadcast comparisons and move in one shuffle; more go through the bitonic
-// network. Both give the same lanes.
-__device__ __forceinline__ void warp_sort_kept(uint64_t& x, uint32_t& f, unsigned kb) {
-  const int nk = __popc(kb);
-  if (nk > 4) {
-    warp_sort_asc_payload(x, f);
-    return;
-  }
+// The same for the lanes in kb, by the whole warp: 32 equally spaced entries are read
+// once; then every key takes a ballot over them and one over the stretch it falls into.
+// Lanes outside kb get 0. Used where few lanes hold a key: a per-lane search is a chain
+// of dependent loads, this is two.
+__device__ __forceinline__ int warp_lower_bound(saddr a, int n, uint64_t x, unsigned kb) {
   const int lane = lane_id();
-  const bool mine = (kb >> lane) & 1u;
+  const int step = (n + 31) >> 5;
+  const int li = (lane + 1) * step - 1;
+  const uint64_t sample = li < n ? lds64(a + 8 * li) : kKeyMax;
   int rank = 0;
+#pragma unroll 1
   for (unsigned rest = kb; rest; rest &= rest - 1) {
-    const uint64_t y = __shfl_sync(kFull, x, __ffs(rest) - 1);
-    rank += y < x;
+    const int src = __ffs(rest) - 1;
+    const uint64_t y = __shfl_sync(kFull, x, src);
+    int at = __popc(__ballot_sync(kFull, sample < y)) * step;  // whole stretches below y
+    const int end = at + step - 1 < n ? at + step - 1 : n;     // entry at + step - 1 is not below y
+#pragma unroll 1
+    for (int b = at; b < end; b += 32) at += __popc(__ballot_sync(kFull, b + lane < end && lds64(a + 8 * (b + lane)) < y));
+    if (lane == src) rank = at;
   }
-  int src = lane;
-  for (int r = 0; r < nk; ++r) {
-    const unsigned b = __ballot_sync(kFull, mine && rank == r);
-    if (lane == r) src = __ffs(b) - 1;
-  }
-  const uint64_t y = __shfl_sync(kFull, x, src);
-  const uint32_t g = __shfl_sync(kFull, f, src);
-  x = lane < nk ? y : kKeyMax;
-  f = lane < nk ? g : 0u;
+  return rank;
 }
 
-__device__ __forceinline__ uint64_t warp_sort_kept(uint64_t x, unsigned kb) {
-  uint32_t f = 0;
-  warp_sort_kept(x, f, kb);
-  return x;
+__device__ __forceinline__ bool contains_u64(saddr a, int n, uint64_t x) {
+  const int i = lower_bound_u64(a, n, x);
+  return i < n && lds64(a + 8 * i) == x;
 }
 
-// First index i in a[0, n) with a[i] >= x (per lane).
-__device__ __forceinline__ int lower_bound_u64(const uint64_t* a, int n, uint64_t x) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (a[mid] < x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-// First index i in a[0, n) with a[i] > x (per lane).
-__device__ __forceinline__ int upper_bound_u64(const uint64_t* a, int n, uint64_t x) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (a[mid] <= x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-__device__ __forceinline__ bool contains_u64(const uint64_t* a, int n, uint64_t x) {
-  int i = lower_bound_u64(a, n, x);
-  return i < n && a[i] == x;
-}
-
-// Merges a sorted batch into the sorted array arr[0, n) of capacity cap, in place.
-// Every lane of the warp calls it. Lane i < nb holds the i-th smallest batch key
-// (distinct from every arr entry); the other lanes hold kKeyMax. Entries that fall
-// beyond cap are dropped (the largest ones). flags (may be null) move with their
-// keys; new entries get flag 0. R is 32 ints of per-warp shared scratch. rank, when
-// given (>= 0 on the lanes < nb), is lower_bound(arr, n, bk), already known.
-// Returns the new size; *r0 = rank of the smallest batch key in the old array
-// (entries below r0 did not move); *dropped = some entry fell beyond cap.
-__device__ __forceinline__ int warp_merge(uint64_t* arr, uint8_t* flags, int n, int cap, uint64_t bk,
-                                          int nb, int* R, int* r0_out, bool* dropped, int rank = -1) {
+// Number of entries of the sorted array of n keys at a that are <= x, the same x on every
+// lane: the warp probes 32 equally spaced entries per step.
+__device__ __forceinline__ int warp_count_le(saddr a, int n, uint64_t x) {
   const int lane = lane_id();
-  int r = (lane < nb) ? (rank >= 0 ? rank : lower_bound_u64(arr, n, bk)) : n;
-  R[lane] = r;
-  __syncwarp();
-  const int r0 = __shfl_sync(kFull, r, 0);
-  if (n > 0 && nb > 0) {
-    for (int base = (n - 1) & ~31; base >= (r0 & ~31); base -= 32) {
-      int j = base + lane;
-      bool act = j >= r0 && j < n;
-      uint64_t v = 0;
-      uint8_t f = 0;
-      int dst = 0;
-      if (act) {
-        int a = 0, b = nb;  // number of batch keys with rank <= j
-        while (a < b) {
-          int mid = (a + b) >> 1;
-          if (R[mid] <= j) a = mid + 1; else b = mid;
-        }
-        dst = j + a;
-        v = arr[j];
-        if (flags) f = flags[j];
-      }
-      __syncwarp();
-      if (act && dst < cap) {
-        arr[dst] = v;
-        if (flags) flags[dst] = f;
-      }
-      __syncwarp();
-    }
+  int lo = 0;  // entries below lo are <= x, entries from hi on are > x
+  int hi = n;
+#pragma unroll 1
+  while (hi > lo) {
+    const int step = (hi - lo + 31) >> 5;
+    const int i = lo + (lane + 1) * step - 1;  // the last entry of this lane's stretch
+    const unsigned over = __ballot_sync(kFull, i >= hi || lds64(a + 8 * i) > x);
+    const int f = over ? __ffs(over) - 1 : 32;  // the first stretch that is not wholly <= x
+    const int nlo = lo + f * step;
+    hi = f == 32 ? nlo : (nlo + step - 1 < hi ? nlo + step - 1 : hi);
+    lo = nlo < n ? nlo : n;
+    if (hi < lo) hi = lo;
   }
-  if (lane < nb) {
-    int dst = r + lane;
-    if (dst < cap) {
-      arr[dst] = bk;
-      if (flags) flags[dst] = 0;
-    }
-  }
-  __syncwarp();
-  *r0_out = r0;
-  *dropped = (n + nb) > cap;
-  return (n + nb) < cap ? (n + nb) : cap;
+  return lo;
 }
 
-// Transposed warp reduction of V partial values per lane (V in {2, 4, 8, 16, 32}).
-// Afterwards the lanes whose index >> log2(32/V) equals u hold the sum over all
-// 32 lanes of value u. Every value is summed by the same tree (pairs across lane
-// bit 4, then bit 3, ..., bit 0), so a vector's distance does not depend on the
-// slot it was computed in.
+// Transposed reduction over groups of eight lanes of V partial values per lane (V in
+// {2, 4, 8}): lane 8 g + u * (8 / V) (and the lanes after it, up to the next) ends with
+// value u of its group, summed over pairs of lanes 4, 2 and 1 apart, in this order.
 template <int V>
-__device__ __forceinline__ float warp_transpose_reduce(float (&v)[V]) {
+__device__ __forceinline__ float oct_transpose_reduce(float (&v)[V]) {
   const int lane = lane_id();
-  int off = 16;
+  int off = 4;
 #pragma unroll
   for (int cnt = V; cnt > 1; cnt >>= 1, off >>= 1) {
     const int half = cnt >> 1;
     const bool up = (lane & off) != 0;
 #pragma unroll
     for (int i = 0; i < half; ++i) {
-      float send = up ? v[i] : v[i + half];
-      float keep = up ? v[i + half] : v[i];
+      const float send = up ? v[i] : v[i + half];
+      const float keep = up ? v[i + half] : v[i];
       v[i] = keep + __shfl_xor_sync(kFull, send, off);
     }
   }
@@ -201,38 +149,53 @@ __device__ __forceinline__ float warp_transpose_reduce(float (&v)[V]) {
   return v[0];
 }
 
-// Vector storage formats. A row is dp4 chunks of 4 elements; lane L handles chunks
-// L, L + 32, ... in every format, so the query registers and the reduction tree
-// are the same and only the load width differs (16, 8 or 4 bytes per chunk).
+// Vector storage formats. A row is dp4 chunks of 4 elements; every format gives a chunk
+// to the same lane, so the reduction tree is the same and only the load width differs
+// (16, 8 or 4 bytes per chunk).
 //
 // Raw is a chunk as loaded (16, 8 or 4 bytes: 4, 2 or 1 registers); decode() turns it
-// into four floats. Distance groups and the pre-filter scan's load batches hold what
-// kHoldRaw says: raw bfloat16 chunks, decoded at use, let a scan batch hold all 32
-// rows of a step in 64 registers; FP8 rows are decoded at load (measured on GB300:
-// raw bfloat16 about 5 % faster on mixed batches, raw FP8 about 6 % slower).
+// into four floats, at use.
+// Read-only loads that leave no line in L1: a row is read once by its warp, and the L1
+// beside a full shared memory is small. Volatile: all loads of a group stay together in
+// front of the arithmetic. Otherwise the compiler moves each into the branch that uses
+// its chunk, and a group costs four memory latencies instead of one.
+__device__ __forceinline__ float4 load_stream16(const void* p) {
+  float4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+      : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint2 load_stream8(const void* p) {
+  uint2 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint32_t load_stream4(const void* p) {
+  uint32_t v;
+  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+
 struct StoreF32 {
   static constexpr int kChunkBytes = 16;
   static constexpr bool kScaled = false;
   using Raw = float4;
   static constexpr int kRawRegs = 4;
-  static constexpr bool kHoldRaw = true;
   __device__ static __forceinline__ Raw load_raw(const unsigned char* row, int c) {
-    return __ldg(reinterpret_cast<const float4*>(row) + c);
+    return load_stream16(row + 16 * c);
   }
   __device__ static __forceinline__ Raw zero_raw() { return make_float4(0.f, 0.f, 0.f, 0.f); }
   __device__ static __forceinline__ float4 decode(const Raw& r) { return r; }
-  __device__ static __forceinline__ float4 load(const unsigned char* row, int c, float) {
-    return __ldg(reinterpret_cast<const float4*>(row) + c);
-  }
+  __device__ static __forceinline__ float4 load(const unsigned char* row, int c, float) { return load_raw(row, c); }
 };
 struct StoreBF16 {  // bfloat16, converted from float32 with round-to-nearest-even
   static constexpr int kChunkBytes = 8;
   static constexpr bool kScaled = false;
   using Raw = uint2;
   static constexpr int kRawRegs = 2;
-  static constexpr bool kHoldRaw = true;
   __device__ static __forceinline__ Raw load_raw(const unsigned char* row, int c) {
-    return __ldg(reinterpret_cast<const uint2*>(row) + c);
+    return load_stream8(row + 8 * c);
   }
   __device__ static __forceinline__ Raw zero_raw() { return make_uint2(0u, 0u); }
   __device__ static __forceinline__ float4 decode(const Raw& u) {
@@ -252,9 +215,8 @@ struct StoreFP8 {
   static constexpr bool kScaled = true;
   using Raw = uint32_t;
   static constexpr int kRawRegs = 1;
-  static constexpr bool kHoldRaw = false;
   __device__ static __forceinline__ Raw load_raw(const unsigned char* row, int c) {
-    return __ldg(reinterpret_cast<const uint32_t*>(row) + c);
+    return load_stream4(row + 4 * c);
   }
   __device__ static __forceinline__ Raw zero_raw() { return 0u; }
   __device__ static __forceinline__ float4 decode(const Raw& u) {
@@ -269,14 +231,8 @@ struct StoreFP8 {
   }
 };
 
-// A chunk as a distance group holds it (raw, or decoded at load) and its value.
 template <class T>
-using Held = typename std::conditional<T::kHoldRaw, typename T::Raw, float4>::type;
-template <class T>
-__device__ __forceinline__ float4 unhold(const Held<T>& h) {
-  if constexpr (T::kHoldRaw) return T::decode(h);
-  else return h;
-}
+using Held = typename T::Raw;  // a chunk as distance groups and the scan hold it
 
 // q - x for a chunk loaded by T::load: for scaled formats x holds codes and the
 // difference is q - scale * code, fused.
@@ -290,6 +246,26 @@ __device__ __forceinline__ float4 diff4(const float4& q, const float4& x, float 
   }
 }
 
+// acc + sum (q - x)^2 over a chunk, element by element in one chain; the differences of
+// unscaled formats are taken two at a time (packed float32, the same rounding).
+template <class T>
+__device__ __forceinline__ float sum_sq(const float4& q, const float4& x, float scale, float acc) {
+  float4 e;
+  if constexpr (T::kScaled) {
+    e = diff4<T>(q, x, scale);
+  } else {
+    asm("{\n .reg .b64 q0, q1, x0, x1;\n mov.b64 q0, {%4, %5};\n mov.b64 q1, {%6, %7};\n mov.b64 x0, {%8, %9};\n"
+        " mov.b64 x1, {%10, %11};\n sub.rn.f32x2 q0, q0, x0;\n sub.rn.f32x2 q1, q1, x1;\n mov.b64 {%0, %1}, q0;\n"
+        " mov.b64 {%2, %3}, q1;\n}"
+        : "=f"(e.x), "=f"(e.y), "=f"(e.z), "=f"(e.w)
+        : "f"(q.x), "f"(q.y), "f"(q.z), "f"(q.w), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w));
+  }
+  acc = fmaf(e.x, e.x, acc);
+  acc = fmaf(e.y, e.y, acc);
+  acc = fmaf(e.z, e.z, acc);
+  return fmaf(e.w, e.w, acc);
+}
+
 // The value of a chunk loaded by T::load (the scale applied for scaled formats).
 template <class T>
 __device__ __forceinline__ float4 value4(const float4& x, float scale) {
@@ -297,38 +273,14 @@ __device__ __forceinline__ float4 value4(const float4& x, float scale) {
   else return x;
 }
 
-// Squared-L2 partial of one lane over its chunks of a row in storage format T.
-template <class T, int CH>
-__device__ __forceinline__ float l2_partial_t(const float4 (&q)[CH], const unsigned char* row, int nchunks,
-                                              float scale) {
+// Copies the query (d floats, any alignment) into qs, dp4 float4 chunks of shared
+// memory, zero beyond d. Called by a whole warp, which may read qs afterwards.
+__device__ __forceinline__ void load_query(float4* qs, const float* qrow, int d, int dp4) {
   const int lane = lane_id();
-  float s = 0.f;
-#pragma unroll
-  for (int t = 0; t < CH; ++t) {
-    int c = lane + 32 * t;
-    if (c < nchunks) {
-      const float4 e = diff4<T>(q[t], T::load(row, c, scale), scale);
-      s = fmaf(e.x, e.x, s);
-      s = fmaf(e.y, e.y, s);
-      s = fmaf(e.z, e.z, s);
-      s = fmaf(e.w, e.w, s);
-    }
-  }
-  return s;
-}
-
-// Loads the query into the per-lane chunks (zero beyond d).
-template <int CH>
-__device__ __forceinline__ void load_query(float4 (&q)[CH], const float* qrow, int d) {
-  const int lane = lane_id();
-#pragma unroll
-  for (int t = 0; t < CH; ++t) {
-    int c = (lane + 32 * t) * 4;
-    q[t].x = c + 0 < d ? qrow[c + 0] : 0.f;
-    q[t].y = c + 1 < d ? qrow[c + 1] : 0.f;
-    q[t].z = c + 2 < d ? qrow[c + 2] : 0.f;
-    q[t].w = c + 3 < d ? qrow[c + 3] : 0.f;
-  }
+  float* f = reinterpret_cast<float*>(qs);
+  __syncwarp();
+  for (int c = lane; c < 4 * dp4; c += 32) f[c] = c < d ? __ldg(qrow + c) : 0.f;
+  __syncwarp();
 }
 
 }  // namespace unify

@@ -167,9 +167,25 @@ __global__ void lowp_kernel(const float* __restrict__ vec, const int32_t* __rest
   }
 }
 
+// Bitmap-marked neighbours of every row in slot order, the first GW of them (-1 past the
+// end, and for marks beyond the row's slots): a post-filter expansion then reads GW
+// consecutive ids instead of W bitmap words and as many scattered ones.
+__global__ void marked_kernel(const int32_t* __restrict__ adj, const uint32_t* __restrict__ gmask, int64_t rows, int W,
+                              int SM, int GW, int32_t* __restrict__ out) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rows; i += (int64_t)gridDim.x * blockDim.x) {
+    int c = 0;
+    for (int w = 0; w < W && c < GW; ++w)
+      for (uint32_t m = gmask[i * W + w]; m != 0 && c < GW; m &= m - 1) {
+        const int slot = 32 * w + __ffs(m) - 1;
+        out[i * GW + c++] = slot < SM ? adj[i * SM + slot] : -1;
+      }
+    for (; c < GW; ++c) out[i * GW + c] = -1;
+  }
+}
+
 void free_device(DeviceIndex& ix) {
   void* ptrs[] = {ix.vec, ix.vec_sorted, ix.sorted_ids, ix.sorted_attr, ix.pos, ix.upper_base, ix.adj0,
-                  ix.gmask0, ix.adjU, ix.gmaskU, ix.seg_bounds, ix.seg_start, ix.vt_bf16, ix.vts_bf16,
+                  ix.gadj0, ix.adjU, ix.gadjU, ix.seg_bounds, ix.seg_start, ix.vt_bf16, ix.vts_bf16,
                   ix.vt_fp8, ix.vts_fp8, ix.scale_fp8, ix.scale_fp8_sorted, ix.xn_bf16_sorted,
                   ix.xn_f32_sorted, ix.xn_fp8_sorted};
   for (void* p : ptrs)
@@ -179,7 +195,7 @@ void free_device(DeviceIndex& ix) {
   ix.vec = ix.vec_sorted = nullptr;
   ix.sorted_ids = ix.pos = ix.upper_base = ix.adj0 = ix.adjU = ix.seg_start = nullptr;
   ix.sorted_attr = ix.seg_bounds = nullptr;
-  ix.gmask0 = ix.gmaskU = nullptr;
+  ix.gadj0 = ix.gadjU = nullptr;
 }
 
 template <typename T>
@@ -353,9 +369,31 @@ extern "C" int unify_load_index(const char* path, int device, unify_index_t** ou
   if (e == cudaSuccess) e = cudaMemcpy(ix.sorted_ids, sorted_ids, n * sizeof(int32_t), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = upload(&ix.upper_base, upper_base, n);
   if (e == cudaSuccess) e = upload(&ix.adj0, adj0, n * SM);
-  if (e == cudaSuccess) e = upload(&ix.gmask0, gmask0, n * ix.W);
   if (e == cudaSuccess) e = upload(&ix.adjU, adjU, nu * SM);
-  if (e == cudaSuccess) e = upload(&ix.gmaskU, gmaskU, nu * ix.W);
+  // marked neighbours: at most 64 of a row are followed
+  uint32_t* d_gmask = nullptr;
+  int marked = 1;
+  for (int part = 0; part < 2; ++part) {
+    const uint32_t* gm = part == 0 ? gmask0 : gmaskU;
+    for (uint64_t r = 0; r < (part == 0 ? n : nu); ++r) {
+      int c = 0;
+      for (int w = 0; w < ix.W; ++w) c += __builtin_popcount(gm[r * ix.W + w]);
+      marked = c > marked ? c : marked;
+    }
+  }
+  ix.GW = ((marked < 64 ? marked : 64) + 3) & ~3;
+  for (int part = 0; part < 2; ++part) {
+    const uint64_t rows = part == 0 ? n : nu;
+    int32_t** dst = part == 0 ? &ix.gadj0 : &ix.gadjU;
+    if (e == cudaSuccess) e = upload(&d_gmask, part == 0 ? gmask0 : gmaskU, rows * ix.W);
+    if (e == cudaSuccess) e = cudaMalloc(dst, rows * ix.GW * sizeof(int32_t));
+    if (e == cudaSuccess) {
+      marked_kernel<<<1024, 256>>>(part == 0 ? ix.adj0 : ix.adjU, d_gmask, (int64_t)rows, ix.W, (int)SM, ix.GW, *dst);
+      e = cudaGetLastError();
+    }
+    if (d_gmask) cudaFree(d_gmask);
+    d_gmask = nullptr;
+  }
   if (e == cudaSuccess) e = upload(&ix.seg_bounds, ix.h_seg_bounds, (uint64_t)ix.S + 1);
   if (e == cudaSuccess) e = upload(&ix.seg_start, ix.h_seg_start, (uint64_t)ix.S + 1);
   if (e == cudaSuccess) e = cudaMalloc(&ix.vec_sorted, n * ix.dp * sizeof(float));

@@ -34,9 +34,12 @@ struct DeviceIndex {
   int32_t* pos = nullptr;       // (n) position of each id in attribute order
   int32_t* upper_base = nullptr;
   int32_t* adj0 = nullptr;      // (n, S, M), -1 padded
-  uint32_t* gmask0 = nullptr;   // (n, W)
   int32_t* adjU = nullptr;      // (n_upper, S, M)
-  uint32_t* gmaskU = nullptr;   // (n_upper, W)
+  // bitmap-marked neighbours, compacted in slot order (-1 past the end): the first GW
+  // marked slots of every row
+  int GW = 0;                   // the largest number of marked slots of a row, at most 64, rounded up to 4
+  int32_t* gadj0 = nullptr;     // (n, GW)
+  int32_t* gadjU = nullptr;     // (n_upper, GW)
   int64_t* seg_bounds = nullptr;  // (S+1)
   int32_t* seg_start = nullptr;   // (S+1)
   // reduced-precision copies (rows of dp/4 chunks of 4 elements): by id and in attribute order

@@ -943,12 +943,15 @@ __global__ void tc_bound(TcArgs a) {
 // an exact warp scan of
 // its range instead: the stored rows (format T) against the float32 query, direct
 // differences, the same selection as the warp scan of the search kernel. After a
-// timed-out wait the rows are empty and flagged.
+// timed-out wait the rows are empty and flagged. Bound by the gathers of the re-rank (R
+// float32 rows per query, scattered); G rows of up to two blocks of 128 elements are in
+// flight per warp, and 128 registers keep 16 warps per SM.
 template <class T, int CH, int G>
-__global__ void __launch_bounds__(128) tc_finish(TcArgs a) {
+__global__ void __launch_bounds__(128, 4) tc_finish(TcArgs a) {
+  __shared__ float4 qv[4][32 * CH];
+  __shared__ __align__(16) uint64_t SK[4][32];
   __shared__ uint64_t top[4][kTcRMax];
   __shared__ uint64_t out[4][kTcRMax];
-  __shared__ int R[4][32];
   __shared__ int clist[4][32];
   const int warp = threadIdx.x >> 5, lane = lane_id();
   const int nA = a.counters[CNT_QA];
@@ -957,8 +960,7 @@ __global__ void __launch_bounds__(128) tc_finish(TcArgs a) {
   for (int pos = blockIdx.x * 4 + warp; pos < nA; pos += warps) {
     const int qi = a.aq[pos];
     const int pa = a.pa[qi], pb = a.pb[qi];
-    float4 qv[CH];
-    load_query<CH>(qv, a.q + (int64_t)qi * a.d, a.d);
+    load_query(qv[warp], a.q + (int64_t)qi * a.d, a.d, a.dp4);
     const int c = a.qcnt[pos];
     const bool overflow = c > kTcQCap;
     int nt = 0;
@@ -968,22 +970,22 @@ __global__ void __launch_bounds__(128) tc_finish(TcArgs a) {
       const uint64_t* src = a.qlist + (int64_t)pos * kTcQCap;
       for (int off = 0; off < c; off += 32) {
         const uint64_t key = off + lane < c ? src[off + lane] : kKeyMax;
-        nt = topk_offer(top[warp], nt, a.R, key, R[warp]);
+        nt = topk_offer(sa(top[warp]), nt, a.R, key, sa(SK[warp]));
       }
     } else {
       for (int base = pa; base < pb; base += 32) {
         int cid = base + lane < pb ? __ldg(a.sorted_ids + base + lane) : -1;
-        const float dist = batch_dist<T, CH, G>(qv, cid, a.vt, a.dp4 * T::kChunkBytes, a.vscale, a.dp4, clist[warp]);
-        nt = topk_offer(top[warp], nt, a.R, cid >= 0 ? make_key(dist, cid) : kKeyMax, R[warp]);
+        const float dist = batch_dist<T, CH, G>(sa(qv[warp]), cid, a.vt, a.dp4 * T::kChunkBytes, a.vscale, a.dp4, sa(clist[warp]));
+        nt = topk_offer(sa(top[warp]), nt, a.R, cid >= 0 ? make_key(dist, cid) : kKeyMax, sa(SK[warp]));
       }
     }
     int no = 0;
     for (int off = 0; off < nt; off += 32) {
       int cid = off + lane < nt ? key_id(top[warp][off + lane]) : -1;
       if (cid >= a.n) cid = -1;
-      const float dist = batch_dist<StoreF32, CH, G>(qv, cid, reinterpret_cast<const unsigned char*>(a.vec),
-                                                     a.dp4 * 16, nullptr, a.dp4, clist[warp]);
-      no = topk_offer(out[warp], no, a.k, cid >= 0 ? make_key(dist, cid) : kKeyMax, R[warp]);
+      const float dist = batch_dist<StoreF32, CH, G>(sa(qv[warp]), cid, reinterpret_cast<const unsigned char*>(a.vec),
+                                                     a.dp4 * 16, nullptr, a.dp4, sa(clist[warp]));
+      no = topk_offer(sa(out[warp]), no, a.k, cid >= 0 ? make_key(dist, cid) : kKeyMax, sa(SK[warp]));
     }
     write_row(out[warp], no, a.k, qi, a.o);
     if (lane == 0) {
@@ -1202,9 +1204,9 @@ cudaError_t launch_tc(const DeviceIndex& ix, const Scratch& sc, const float* q, 
   else if (ch <= 2)
     tc_finish<T, 2, 8><<<fgrid, 128, 0, st>>>(a);
   else if (ch <= 4)
-    tc_finish<T, 4, 4><<<fgrid, 128, 0, st>>>(a);
+    tc_finish<T, 4, 8><<<fgrid, 128, 0, st>>>(a);
   else
-    tc_finish<T, 8, 2><<<fgrid, 128, 0, st>>>(a);
+    tc_finish<T, 8, 8><<<fgrid, 128, 0, st>>>(a);
   return cudaGetLastError();
 }
 
