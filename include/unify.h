@@ -95,7 +95,8 @@ typedef struct {
   int visited_cap;     /* visited-filter slots per query, power of two, default 2048 */
   int max_expansions;  /* expansions per layer before UNIFY_Q_LIMIT, default 100000 */
   int warps_per_block; /* search warps per CTA (one query or scan item each), 1..4, default 4 */
-  int scan_rows;       /* pre-filter rows per scan work item, default 8192 */
+  int scan_rows;       /* pre-filter rows per scan work item, at most (smaller batches are cut
+                          finer), default 8192 */
   int reg_budget;      /* build of the search kernel for rows of up to 128 elements: 128 (128 registers
                           per thread, 16 warps per SM), 80 (96 registers, 20 warps) or 64 (80
                           registers, 24 warps; the smaller builds hold fewer rows in flight per

@@ -305,7 +305,8 @@ int run_search(unify_index_t* idx, const float* q, const int64_t* lo, const int6
   {
     NvtxRange r("unify:route");
     PhaseTimer t(idx->tm, 0, st);
-    e = launch_route(idx->ix, sc, lo, hi, nq, p.tau_a, p.tau_b, strategy, p.scan_rows, 1, sc.pa, sc.pb, sc.mask,
+    e = launch_route(idx->ix, sc, lo, hi, nq, p.tau_a, p.tau_b, strategy,
+                     scan_item_rows(idx->ix, p, nq, strategy), 1, sc.pa, sc.pb, sc.mask,
                      sc.strat, &o, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "route kernel");

@@ -15,7 +15,9 @@ namespace unify {
 constexpr int kMaxS = 32;      // segments (one bit each in a 32-bit mask)
 constexpr int kMaxK = 256;     // results per query
 constexpr int kMaxCand = 4096; // candidate buffer entries per query
-constexpr int kMaxScanBlocks = 64;  // scan work items per pre-filter query
+constexpr int kMaxScanBlocks = 64;  // scan work items per query of capacity that the scratch holds room for; a
+                                    // batch below the capacity shares them (launch_route)
+constexpr int kMaxItemsPerQuery = 1024;
 
 // Device-resident index. Arrays marked (n) are indexed by object id unless noted.
 struct DeviceIndex {
@@ -161,6 +163,7 @@ size_t tc_query_row_bytes(int d);  // bytes of one query row of the tensor-core 
 cudaError_t launch_tcscan(const DeviceIndex& ix, const Scratch& sc, const float* q, int64_t nq, const Params& p,
                           const Outputs& o, cudaStream_t st);
 int batch_smem_per_warp(const Params& p);
+int scan_item_rows(const DeviceIndex& ix, const Params& p, int64_t nq, int strategy);  // rows per scan work item of this batch
 int rerank_count(const Params& p);  // candidates re-ranked in FP32 (0 for FP32 storage)
 
 void set_error(const std::string& msg);

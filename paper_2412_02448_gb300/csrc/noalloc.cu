@@ -126,7 +126,8 @@ extern "C" int unify_search_noalloc(unify_index_t* idx, const float* q, const in
   cudaError_t e = cudaMemsetAsync(sc.counters, 0, kNumCounters * sizeof(int32_t), st);
   if (e != cudaSuccess) return cuda_fail(e, "counter reset");
   Outputs o{out_ids, out_dist, out_count, out_status, nullptr};
-  e = launch_route(idx->ix, sc, lo, hi, nq, prm.tau_a, prm.tau_b, st_code, prm.scan_rows, 1, sc.pa, sc.pb,
+  e = launch_route(idx->ix, sc, lo, hi, nq, prm.tau_a, prm.tau_b, st_code,
+                   scan_item_rows(idx->ix, prm, nq, st_code), 1, sc.pa, sc.pb,
                    sc.mask, sc.strat, &o, st);
   if (e != cudaSuccess) return cuda_fail(e, "route kernel");
   e = launch_batch(idx->ix, sc, q, prm, o, st);

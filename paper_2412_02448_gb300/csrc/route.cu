@@ -39,6 +39,7 @@ struct RouteArgs {
   int64_t tau_a, tau_b;
   int forced;        // -1: range-aware, else the strategy for every query
   int scan_rows;
+  int max_items;     // scan work items per query, at most (the scratch's share of this batch)
   int build_queues;
   int32_t* pa;
   int32_t* pb;
@@ -93,7 +94,7 @@ __global__ void route_kernel(RouteArgs a, const int64_t* __restrict__ seg_bounds
   if (st == UNIFY_PRE) {
     int64_t nb = (Y + a.scan_rows - 1) / a.scan_rows;
     if (nb < 1) nb = 1;
-    if (nb > kMaxScanBlocks) nb = kMaxScanBlocks;
+    if (nb > a.max_items) nb = a.max_items;
     int base = atomicAdd(&a.counters[CNT_ITEMS], (int)nb);
     a.nblk[i] = (int)nb;
     a.qbase[i] = base;
@@ -123,6 +124,12 @@ cudaError_t launch_route(const DeviceIndex& ix, const Scratch& sc, const int64_t
   a.tau_b = tau_b;
   a.forced = forced;
   a.scan_rows = scan_rows > 0 ? scan_rows : 8192;
+  // items and partial lists of cap_nq * kMaxScanBlocks work items, shared by nq <= cap_nq queries
+  a.max_items = kMaxScanBlocks;
+  if (build_queues && nq > 0) {
+    const int64_t share = sc.cap_nq * kMaxScanBlocks / nq;
+    a.max_items = (int)(share < kMaxItemsPerQuery ? share : kMaxItemsPerQuery);
+  }
   a.build_queues = build_queues;
   a.pa = out_pa;
   a.pb = out_pb;

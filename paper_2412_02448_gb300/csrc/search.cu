@@ -4,6 +4,29 @@
 
 namespace unify {
 
+// Rows per scan work item, at most p.scan_rows. An item is one warp's, so it is the
+// granularity of the batch's tail and, when there are few queries, all the parallelism
+// there is: with fewer queries than resident warps (16 per SM) it shrinks in proportion,
+// from 1 MB of float32 rows down to 64 KB, and it grows with the batch up to 4 MB; never
+// below 64 rows, nor below 4 rows per key kept (each item sorts its own list of the kept
+// keys, which the query's last item merges). In a routed batch the graph walks hold most
+// warps for longer than a 4 MB item takes, so that finer items only take issue slots from
+// them (2 % slower at 1,003 queries): there a batch counts sixteenfold.
+// Measured on GB300 against items of 8,192 rows: 17 queries over 15,000 rows of 512 B
+// each 585 -> 63 us; 301 queries over 4,200 rows of 3,840 B 4,900 -> 928 us.
+int scan_item_rows(const DeviceIndex& ix, const Params& p, int64_t nq, int strategy) {
+  const int64_t row_bytes = (int64_t)ix.dp * 4;  // a row's arithmetic is the same in every storage format
+  const int64_t slots = 16ll * ix.num_sms;
+  int64_t bytes = (1ll << 20) * (strategy == UNIFY_AUTO ? 16 : 1) * nq / slots;
+  if (bytes < (64 << 10)) bytes = 64 << 10;
+  if (bytes > (4 << 20)) bytes = 4 << 20;
+  const int64_t kept = rerank_count(p) > p.k ? rerank_count(p) : p.k;
+  int64_t rows = bytes / row_bytes;
+  if (rows < 64) rows = 64;
+  if (rows < 4 * kept) rows = 4 * kept;
+  return (int)(rows < p.scan_rows ? rows : p.scan_rows);
+}
+
 int rerank_count(const Params& p) { return p.dtype == UNIFY_FP32 ? 0 : p.rerank_mult * p.k; }
 
 int batch_ann_cap(const Params& p) {

@@ -630,6 +630,30 @@ __device__ __forceinline__ void graph_query(const BatchArgs& a, const WarpMem& w
   __syncwarp();
 }
 
+// The kk smallest keys of nb ascending lists of kk keys each, into ann; returns how many.
+// Each lane walks one list from its front and stops at the first key that cannot enter
+// any more, the next key of its list already in flight.
+static __device__ __noinline__ int merge_lists(saddr off, const uint64_t* lists, int nb, int kk) {
+  const WarpMem w{off, shared_args()};
+  const saddr topk = w.ann();
+  const int lane = lane_id();
+  int nt = 0;
+  for (int b0 = 0; b0 < nb; b0 += 32) {
+    bool has = b0 + lane < nb;
+    const unsigned long long* list =
+        reinterpret_cast<const unsigned long long*>(lists) + (int64_t)(has ? b0 + lane : 0) * kk;
+    uint64_t next = has ? __ldcg(list) : kKeyMax;
+    for (int t = 0; t < kk; ++t) {
+      const uint64_t key = next;
+      next = has && t + 1 < kk ? __ldcg(list + t + 1) : kKeyMax;
+      has = has && key < (nt >= kk ? lds64(topk + 8 * (kk - 1)) : kKeyMax);
+      if (!__any_sync(kFull, has)) break;
+      nt = topk_offer(topk, nt, kk, has ? key : kKeyMax, w.SK());
+    }
+  }
+  return nt;
+}
+
 template <class T, int CH, int RB, int GF>
 __device__ __noinline__ void scan_item(uint32_t off, int it) {
   const BatchArgs& a = shared_args();
@@ -715,15 +739,7 @@ __device__ __noinline__ void scan_item(uint32_t off, int it) {
       return;
     }
     __threadfence();
-    const uint64_t* src = a.part + (int64_t)a.qbase[qi] * kk;
-    const int total = nb * kk;
-    nt = 0;
-    for (int t0 = 0; t0 < total; t0 += 32) {
-      const uint64_t key = (t0 + lane < total)
-                               ? __ldcg(reinterpret_cast<const unsigned long long*>(src) + t0 + lane)
-                               : kKeyMax;
-      nt = topk_offer(topk, nt, kk, key, w.SK());
-    }
+    nt = merge_lists(off, a.part + (int64_t)a.qbase[qi] * kk, nb, kk);
     nt = min(nt, Y);
   }
   int cnt;
