@@ -719,9 +719,9 @@ def run(args):
             "cuda_graph": {"ms_per_step": graph_ms, "value": world * nq / (graph_ms / 1000.0),
                            "same_ids_as_direct": graph_ok},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-            # per step: route and search kernels, plus the tensor-core scan's eight
-            # (bucket count, bucket scan, scatter, tile prep, unit plan, two passes, finish)
-            "gpu_launches": (2 + (8 if m32["tc_used"] else 0)) * args.steps,
+            # per step: route and search kernels, plus the tensor-core scan's seven
+            # (scatter, span scan, placement, two passes, bound, finish)
+            "gpu_launches": (2 + (7 if m32["tc_used"] else 0)) * args.steps,
             "other_scan": headline_other,
             "clocks": clk,
             "cpu_baseline": cpu,

@@ -68,7 +68,6 @@ void free_tc(Scratch& sc) {
   release(sc.tc_qlist);
   release(sc.tc_qcnt);
   release(sc.tc_thr);
-  release(sc.tc_sumy);
   release(sc.tc_stage);
   sc.tc_stage_sms = 0;
   sc.tc_rows = 0;
@@ -151,7 +150,6 @@ cudaError_t ensure_tc_scratch(Scratch& sc, int64_t nq, int d, int64_t n, int sms
   if (e == cudaSuccess) e = alloc(sc.tc_qlist, (size_t)rows * kTcQCap);
   if (e == cudaSuccess) e = alloc(sc.tc_qcnt, rows);
   if (e == cudaSuccess) e = alloc(sc.tc_thr, rows);
-  if (e == cudaSuccess) e = alloc(sc.tc_sumy, 1);
   if (e == cudaSuccess) e = alloc(sc.tc_stage, (size_t)sms * kTcEpiThreads * kTcStage);
   if (e != cudaSuccess) {
     free_tc(sc);
@@ -307,7 +305,7 @@ int run_search(unify_index_t* idx, const float* q, const int64_t* lo, const int6
     PhaseTimer t(idx->tm, 0, st);
     e = launch_route(idx->ix, sc, lo, hi, nq, p.tau_a, p.tau_b, strategy,
                      scan_item_rows(idx->ix, p, nq, strategy), 1, sc.pa, sc.pb, sc.mask,
-                     sc.strat, &o, st);
+                     sc.strat, &o, st, tc);
   }
   if (e != cudaSuccess) return cuda_fail(e, "route kernel");
   if (tc) {
@@ -316,7 +314,8 @@ int run_search(unify_index_t* idx, const float* q, const int64_t* lo, const int6
     e = launch_tcscan(idx->ix, sc, q, nq, p, o, st);
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core pre-filter scan");
   }
-  {
+  // with every query in the tensor-core scan the search kernel has nothing to do
+  if (!(tc && strategy == UNIFY_PRE)) {
     NvtxRange r("unify:search kernel");
     PhaseTimer t(idx->tm, 1, st);
     e = launch_batch(idx->ix, sc, q, p, o, st, tc, cj);

@@ -86,7 +86,6 @@ struct Scratch {
   uint64_t* tc_qlist = nullptr;  // per query: kTcQCap candidate keys
   int32_t* tc_qcnt = nullptr;    // per query: candidates found
   unsigned long long* tc_thr = nullptr;   // per query: bound key
-  unsigned long long* tc_sumy = nullptr;  // total in-range rows of the pre-filter queries
   uint64_t* tc_stage = nullptr;  // per scan CTA and epilogue thread: kTcStage keys of the current unit
   int tc_stage_sms = 0;
   int64_t tc_rows = 0;        // query positions (a multiple of 128)
@@ -125,7 +124,8 @@ enum {
   CNT_TC_TAKE_B = 13,                  // next work unit to claim (tensor-core bounding pass)
   CNT_TC_L = 14,                       // span length of the tensor-core scan's tiles (rows)
   CNT_TC_TILES = 15,                   // tiles of the tensor-core scan
-  kNumCounters = 16
+  CNT_TC_SUMY = 16,                    // counters[16..17]: 64-bit total of the pre-filter queries' in-range rows
+  kNumCounters = 18
 };
 
 struct Params {
@@ -155,7 +155,7 @@ struct Outputs {
 cudaError_t launch_route(const DeviceIndex& ix, const Scratch& sc, const int64_t* lo, const int64_t* hi,
                          int64_t nq, int64_t tau_a, int64_t tau_b, int forced, int scan_rows,
                          int build_queues, int32_t* out_pa, int32_t* out_pb, uint32_t* out_mask,
-                         int32_t* out_strat, const Outputs* outs, cudaStream_t st);
+                         int32_t* out_strat, const Outputs* outs, cudaStream_t st, bool tc = false);
 cudaError_t launch_batch(const DeviceIndex& ix, const Scratch& sc, const float* q, const Params& p,
                          const Outputs& o, cudaStream_t st, bool skip_scan = false, const Conj* cj = nullptr);
 bool tc_scan_available(const DeviceIndex& ix, const Params& p);

@@ -64,6 +64,10 @@ struct RouteArgs {
   int32_t* counters;
   int32_t* out_count;     // may be null (set 0 for empty pre-filter queries handled here)
   int32_t* out_counters;  // may be null
+  // tensor-core scan: its tables to clear (slots to -1, spans to 0); null without it
+  int32_t* tc_slotpos;
+  int32_t* tc_spans;
+  int64_t tc_slots, tc_spans_n;
 };
 
 // One warp per query finds its bounds, mask and strategy; then the CTA's first warp takes
@@ -73,11 +77,17 @@ struct RouteArgs {
 // searches before): 5,000 queries 18 -> 8 us.
 __global__ void __launch_bounds__(32 * kRouteWarps) route_kernel(RouteArgs a, const int64_t* __restrict__ seg_bounds,
                                                                  const int32_t* __restrict__ seg_start) {
-  __shared__ int s_strat[kRouteWarps], s_nb[kRouteWarps], s_base[kRouteWarps];
+  __shared__ int s_strat[kRouteWarps], s_nb[kRouteWarps], s_base[kRouteWarps], s_rows[kRouteWarps];
   const int warp = threadIdx.x >> 5, lane = lane_id();
   const int64_t i = (int64_t)blockIdx.x * kRouteWarps + warp;
   const bool valid = i < a.nq;
   int st = -1, nb = 0, Y = 0;
+  if (a.tc_slotpos) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t = t0; t < a.tc_slots / 4; t += stride)  // tc_slots is a multiple of 128
+      reinterpret_cast<int4*>(a.tc_slotpos)[t] = make_int4(-1, -1, -1, -1);
+    for (int64_t t = t0; t < a.tc_spans_n; t += stride) a.tc_spans[t] = 0;
+  }
   if (valid) {
     const int64_t lo = a.lo[i], hi = a.hi[i];
     const int p = half_warp_bound(a.sorted_attr, (int)a.n, lane < 16 ? lo : hi, lane < 16);
@@ -110,6 +120,7 @@ __global__ void __launch_bounds__(32 * kRouteWarps) route_kernel(RouteArgs a, co
   if (lane == 0) {
     s_strat[warp] = st;
     s_nb[warp] = nb;
+    s_rows[warp] = Y;
   }
   __syncthreads();
   if (warp == 0) {
@@ -135,6 +146,11 @@ __global__ void __launch_bounds__(32 * kRouteWarps) route_kernel(RouteArgs a, co
     const int total = __shfl_sync(kFull, incl, kRouteWarps - 1);
     if (lane == 0 && total > 0) base = atomicAdd(&a.counters[CNT_ITEMS], total);
     base = __shfl_sync(kFull, base, 0) + incl - qnb;
+    if (a.tc_slotpos) {
+      const unsigned y = qst == UNIFY_PRE ? (unsigned)s_rows[lane] : 0u;
+      const unsigned long long sum = __reduce_add_sync(kFull, y & 0xffffu) + ((unsigned long long)__reduce_add_sync(kFull, y >> 16) << 16);
+      if (lane == 0 && sum > 0) atomicAdd(reinterpret_cast<unsigned long long*>(a.counters + CNT_TC_SUMY), sum);
+    }
     if (qst == UNIFY_PRE) {
       s_base[lane] = base;
       a.nblk[qi] = qnb;
@@ -157,7 +173,7 @@ __global__ void __launch_bounds__(32 * kRouteWarps) route_kernel(RouteArgs a, co
 cudaError_t launch_route(const DeviceIndex& ix, const Scratch& sc, const int64_t* lo, const int64_t* hi,
                          int64_t nq, int64_t tau_a, int64_t tau_b, int forced, int scan_rows,
                          int build_queues, int32_t* out_pa, int32_t* out_pb, uint32_t* out_mask,
-                         int32_t* out_strat, const Outputs* outs, cudaStream_t st) {
+                         int32_t* out_strat, const Outputs* outs, cudaStream_t st, bool tc) {
   RouteArgs a;
   a.sorted_attr = ix.sorted_attr;
   a.n = ix.n;
@@ -189,6 +205,10 @@ cudaError_t launch_route(const DeviceIndex& ix, const Scratch& sc, const int64_t
   a.counters = sc.counters;
   a.out_count = outs ? outs->count : nullptr;
   a.out_counters = outs ? outs->counters : nullptr;
+  a.tc_slotpos = tc ? sc.tc_slotpos : nullptr;
+  a.tc_slots = sc.tc_slots;
+  a.tc_spans = sc.tc_spans;
+  a.tc_spans_n = sc.tc_spans_cap;
   if (nq == 0) return cudaSuccess;
   const int64_t blocks = (nq + kRouteWarps - 1) / kRouteWarps;
   route_kernel<<<(unsigned)blocks, 32 * kRouteWarps, 0, st>>>(a, ix.seg_bounds, ix.seg_start);

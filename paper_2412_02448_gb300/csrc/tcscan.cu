@@ -311,7 +311,6 @@ struct TcArgs {
   uint64_t* qlist;      // per query: kTcQCap candidate keys below its bound
   uint64_t* stage;      // per CTA and epilogue thread: kTcStage keys found in the current unit
   int32_t* qcnt;        // per query: candidates found (above kQCap: overflow)
-  unsigned long long* sumy;  // total in-range rows of the pre-filter queries
   unsigned long long* qthr;  // per query: key(T, INT_MAX) of its bound T (kKeyMax: none)
   int64_t slot_cap, span_cap, pcap;  // tile slots, spans and (query, span) pairs the scratch holds
   int32_t* counters;
@@ -337,7 +336,7 @@ __device__ __forceinline__ int unit_tile(const TcArgs& a, int ntiles, int x) {
 // pcap / 64: there are at most P / 128 + ceil(n / L) of them, and
 // L >= 128 n / (pcap - 128) makes ceil(n / L) <= pcap / 128.
 __device__ __forceinline__ int64_t span_len(const TcArgs& a, int nA) {
-  const unsigned long long sy = *a.sumy;
+  const unsigned long long sy = *reinterpret_cast<const unsigned long long*>(a.counters + CNT_TC_SUMY);
   const int64_t room = a.pcap - 2 * (int64_t)nA;  // > 0: pcap is 8 slots per query
   int64_t L = (int64_t)((sy + room - 1) / room);
   const int64_t L2 = (128 * a.n + a.pcap - 129) / (a.pcap - 128);  // pcap >= 1024
@@ -775,32 +774,27 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_scan_kernel(const __grid_con
   }
 }
 
-// Spans of the attribute order met by each pre-filter query: one thread per query
-// position counts itself into every span its range [pa, pb) meets.
-__global__ void tc_span_count(TcArgs a) {
-  const int nA = a.counters[CNT_QA];
-  const int64_t L = span_len(a, nA);
-  if (blockIdx.x == 0 && threadIdx.x == 0) a.counters[CNT_TC_L] = (int)L;
-  for (int pos = blockIdx.x * blockDim.x + threadIdx.x; pos < nA; pos += gridDim.x * blockDim.x) {
-    const int qi = a.aq[pos];
-    const int pa = a.pa[qi], pb = a.pb[qi];
-    if (pb <= pa) continue;
-    for (int64_t sp = pa / L; sp <= (pb - 1) / L; ++sp) atomicAdd(&a.span_cnt[sp], 1);
-  }
-}
-
-// Exclusive prefix sum over the 1024 threads of a CTA; *total gets the sum.
+// Exclusive prefix sum over the 1024 threads of a CTA; *total gets the sum. sm: 33 ints.
 __device__ __forceinline__ int cta_exclusive_scan(int v, int* sm, int* total) {
-  sm[threadIdx.x] = v;
-  __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {
-    const int w = threadIdx.x >= off ? sm[threadIdx.x - off] : 0;
-    __syncthreads();
-    sm[threadIdx.x] += w;
-    __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int incl = v;
+  for (int off = 1; off < 32; off <<= 1) {
+    const int w = __shfl_up_sync(kFull, incl, off);
+    if (lane >= off) incl += w;
   }
-  const int r = sm[threadIdx.x] - v;
-  *total = sm[1023];
+  if (lane == 31) sm[warp] = incl;
+  __syncthreads();
+  if (warp == 0) {
+    int w = sm[lane];
+    for (int off = 1; off < 32; off <<= 1) {
+      const int u = __shfl_up_sync(kFull, w, off);
+      if (lane >= off) w += u;
+    }
+    sm[lane] = w;
+  }
+  __syncthreads();
+  const int r = incl - v + (warp > 0 ? sm[warp - 1] : 0);
+  *total = sm[31];
   __syncthreads();
   return r;
 }
@@ -812,7 +806,7 @@ __device__ __forceinline__ int cta_exclusive_scan(int v, int* sm, int* total) {
 // (all tiles of a span have the same units). Totals go to the counters; tiles past the
 // scratch's slots raise the error flag and are dropped.
 __global__ void tc_span_scan(TcArgs a) {
-  __shared__ int sm[1024];
+  __shared__ int sm[33];
   __shared__ int carry;
   __shared__ unsigned long long blocks;
   const int64_t L = a.counters[CNT_TC_L];
@@ -1004,26 +998,28 @@ __global__ void __launch_bounds__(128, 4) tc_finish(TcArgs a) {
 // the scan's format (zero-padded to dpq elements: bfloat16 by round-to-nearest-even;
 // float32 as given for tf32; E4M3 codes of q / s_q with s_q = max|q| / 448,
 // saturating), the squared norm of those values (for E4M3, of the decoded s_q * code),
-// and its bound, group minima and candidate count reset; its in-range row count is
-// added to the batch's total.
+// its bound, group minima and candidate count reset, and the spans that its range meets
+// counted. (The route kernel summed the batch's in-range rows and cleared the span and
+// slot tables: no memsets, and no launch of its own for the counting.)
 template <int F>
-__global__ void tc_scatter(const int32_t* __restrict__ queues, const int32_t* __restrict__ pa,
-                           const int32_t* __restrict__ pb, const float* __restrict__ q, int d, int dpq,
-                           int32_t* counters, int32_t* aq, float* aqn, float* aqs, void* qb,
-                           unsigned long long* qthr, unsigned* gmin, int32_t* qcnt, unsigned long long* sumy) {
-  const int nA = counters[CNT_QA];
+__global__ void tc_scatter(const int32_t* __restrict__ queues, TcArgs a) {
+  const int nA = a.counters[CNT_QA];
   const int lane = threadIdx.x & 31;
   const int warps = gridDim.x * (blockDim.x >> 5);
+  const int64_t L = span_len(a, nA);
+  const int d = a.d, dpq = a.dpq;
+  void* const qb = a.qb;
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.counters[CNT_TC_L] = (int)L;
   for (int pos = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; pos < nA; pos += warps) {
     const int qi = queues[pos];
-    reinterpret_cast<uint4*>(gmin + (int64_t)pos * 128)[lane] = make_uint4(0x7f800000u, 0x7f800000u, 0x7f800000u,
-                                                                          0x7f800000u);
-    if (lane == 0) {
-      const int y = pb[qi] - pa[qi];
-      if (y > 0) atomicAdd(sumy, (unsigned long long)y);
-      qcnt[pos] = 0;
-    }
-    const float* qrow = q + (int64_t)qi * d;
+    reinterpret_cast<uint4*>(a.gmin + (int64_t)pos * 128)[lane] = make_uint4(0x7f800000u, 0x7f800000u, 0x7f800000u,
+                                                                            0x7f800000u);
+    const int pa = a.pa[qi], pb = a.pb[qi];
+    if (lane == 0) a.qcnt[pos] = 0;
+    if (pb > pa)  // counted into every span its range meets
+      for (unsigned sp = (unsigned)pa / (unsigned)L + lane; sp <= (unsigned)(pb - 1) / (unsigned)L; sp += 32)
+        atomicAdd(&a.span_cnt[sp], 1);
+    const float* qrow = a.q + (int64_t)qi * d;
     float ss = 0.f, sq = 1.f;
     if constexpr (F == kFmtBF16) {
       __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(qb) + (int64_t)pos * dpq;
@@ -1057,10 +1053,10 @@ __global__ void tc_scatter(const int32_t* __restrict__ queues, const int32_t* __
     }
     for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(kFull, ss, off);
     if (lane == 0) {
-      aq[pos] = qi;
-      aqn[pos] = ss;
-      if (aqs) aqs[pos] = sq;
-      qthr[pos] = kKeyMax;
+      a.aq[pos] = qi;
+      a.aqn[pos] = ss;
+      if (a.aqs) a.aqs[pos] = sq;
+      a.qthr[pos] = kKeyMax;
     }
   }
 }
@@ -1153,7 +1149,6 @@ cudaError_t launch_tc(const DeviceIndex& ix, const Scratch& sc, const float* q, 
   a.qlist = sc.tc_qlist;
   a.qcnt = sc.tc_qcnt;
   a.stage = sc.tc_stage;
-  a.sumy = sc.tc_sumy;
   a.qthr = sc.tc_thr;
   a.slot_cap = sc.tc_slots;
   a.span_cap = sc.tc_spans_cap;
@@ -1164,16 +1159,10 @@ cudaError_t launch_tc(const DeviceIndex& ix, const Scratch& sc, const float* q, 
   a.stall = p.tc_scan == 2 ? 1 : 0;
   a.wait_ns = p.tc_scan == 2 ? kTestWaitNs : kWaitNs;
   a.o = o;
-  // queries by position, then spans, tiles, units and slots
-  cudaError_t e = cudaMemsetAsync(sc.tc_sumy, 0, sizeof(unsigned long long), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(sc.tc_spans, 0, (size_t)sc.tc_spans_cap * sizeof(int32_t), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(sc.tc_slotpos, 0xff, (size_t)sc.tc_slots * sizeof(int32_t), st);
-  if (e != cudaSuccess) return e;
-  const int qgrid = (int)std::max<int64_t>(ix.num_sms, (nq + 7) / 8);  // a warp per query, 8 per CTA
-  tc_scatter<F><<<qgrid, 256, 0, st>>>(sc.queues, sc.pa, sc.pb, q, ix.d, dpq, sc.counters, sc.tc_aq, sc.tc_aqn,
-                                       F == kFmtFP8 ? sc.tc_aqs : nullptr, sc.tc_qb, sc.tc_thr, sc.tc_gmin,
-                                       sc.tc_qcnt, sc.tc_sumy);
-  tc_span_count<<<(int)std::max<int64_t>(1, (nq + 255) / 256), 256, 0, st>>>(a);
+  // queries by position and spans, then tiles, units and slots
+  cudaError_t e = cudaSuccess;
+  const int qgrid = (int)std::max<int64_t>(1, (nq + 7) / 8);  // a warp per query, 8 per CTA
+  tc_scatter<F><<<qgrid, 256, 0, st>>>(sc.queues, a);
   tc_span_scan<<<1, 1024, 0, st>>>(a);
   tc_place<<<qgrid, 256, 0, st>>>(a);
   e = cudaGetLastError();
@@ -1198,7 +1187,7 @@ cudaError_t launch_tc(const DeviceIndex& ix, const Scratch& sc, const float* q, 
   // one warp per query of the batch (the pre-filter queries are a part of it), so that
   // every query's list merge and re-rank gathers are in flight at once
   const int ch = (a.dp4 + 31) / 32;
-  const int fgrid = (int)std::max<int64_t>(ix.num_sms * 4, (nq + 3) / 4);
+  const int fgrid = (int)std::max<int64_t>(1, (nq + 3) / 4);
   if (ch <= 1)
     tc_finish<T, 1, 16><<<fgrid, 128, 0, st>>>(a);
   else if (ch <= 2)
