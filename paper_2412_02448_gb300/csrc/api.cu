@@ -305,7 +305,7 @@ int run_search(unify_index_t* idx, const float* q, const int64_t* lo, const int6
     PhaseTimer t(idx->tm, 0, st);
     e = launch_route(idx->ix, sc, lo, hi, nq, p.tau_a, p.tau_b, strategy,
                      scan_item_rows(idx->ix, p, nq, strategy), 1, sc.pa, sc.pb, sc.mask,
-                     sc.strat, &o, st, tc);
+                     sc.strat, &o, &p, st, tc);
   }
   if (e != cudaSuccess) return cuda_fail(e, "route kernel");
   if (tc) {
@@ -481,7 +481,7 @@ extern "C" int unify_route(unify_index_t* idx, const int64_t* lo, const int64_t*
   const int64_t ta = tau_a >= 0 ? tau_a : idx->ix.n / 100;
   const int64_t tb = tau_b >= 0 ? tau_b : idx->ix.n / 2;
   cudaError_t e = launch_route(idx->ix, idx->sc, lo, hi, nq, ta, tb, -1, 8192, 0, out_pa, out_pb, out_mask,
-                               out_strategy, nullptr, (cudaStream_t)stream);
+                               out_strategy, nullptr, nullptr, (cudaStream_t)stream);
   return e == cudaSuccess ? UNIFY_OK : cuda_fail(e, "unify_route");
 }
 

@@ -68,7 +68,8 @@ struct Scratch {
   int32_t* nblk = nullptr;     // scan work items of each pre-filter query
   int32_t* qbase = nullptr;    // index of its first work item
   int32_t* done = nullptr;     // completed scan work items of each pre-filter query
-  int32_t* queues = nullptr;   // 3 x cap_nq: query ids per strategy (A, C, B)
+  int32_t* queues = nullptr;   // 3 x cap_nq: query ids per strategy (A, C, B); C's long walks from its
+                               // front, its short ones from its end
   int2* items = nullptr;       // cap_nq * kMaxScanBlocks scan work items (query, block)
   uint64_t* part = nullptr;    // cap_nq * kMaxScanBlocks * cap_k partial top-k keys
   int32_t* counters = nullptr; // kNumCounters ints, zeroed per call
@@ -117,6 +118,7 @@ enum {
   CNT_QA = 0, CNT_QC = 1, CNT_QB = 2,  // queue lengths
   CNT_ITEMS = 3,                       // scan work items
   CNT_TAKE = 4,                        // head of the combined work queue
+  CNT_QS = 5,                          // short hybrid walks (CNT_QC counts the long ones), see route.cu
   CNT_T0 = 8,                          // counters[8..9]: 64-bit global-timer origin of the search kernel
   CNT_TC_ERR = 10,                     // the tensor-core scan timed out on a wait
   CNT_TC_UNITS = 11,                   // work units of the tensor-core scan
@@ -155,7 +157,7 @@ struct Outputs {
 cudaError_t launch_route(const DeviceIndex& ix, const Scratch& sc, const int64_t* lo, const int64_t* hi,
                          int64_t nq, int64_t tau_a, int64_t tau_b, int forced, int scan_rows,
                          int build_queues, int32_t* out_pa, int32_t* out_pb, uint32_t* out_mask,
-                         int32_t* out_strat, const Outputs* outs, cudaStream_t st, bool tc = false);
+                         int32_t* out_strat, const Outputs* outs, const Params* p, cudaStream_t st, bool tc = false);
 cudaError_t launch_batch(const DeviceIndex& ix, const Scratch& sc, const float* q, const Params& p,
                          const Outputs& o, cudaStream_t st, bool skip_scan = false, const Conj* cj = nullptr);
 bool tc_scan_available(const DeviceIndex& ix, const Params& p);

@@ -128,7 +128,7 @@ extern "C" int unify_search_noalloc(unify_index_t* idx, const float* q, const in
   Outputs o{out_ids, out_dist, out_count, out_status, nullptr};
   e = launch_route(idx->ix, sc, lo, hi, nq, prm.tau_a, prm.tau_b, st_code,
                    scan_item_rows(idx->ix, prm, nq, st_code), 1, sc.pa, sc.pb,
-                   sc.mask, sc.strat, &o, st);
+                   sc.mask, sc.strat, &o, &prm, st);
   if (e != cudaSuccess) return cuda_fail(e, "route kernel");
   e = launch_batch(idx->ix, sc, q, prm, o, st);
   if (e != cudaSuccess) return cuda_fail(e, "search kernel");

@@ -51,6 +51,7 @@ struct RouteArgs {
   int scan_rows;
   int max_items;     // scan work items per query, at most (the scratch's share of this batch)
   int build_queues;
+  int ef_h, ef_p;    // beams of hybrid and post-filter walks
   int32_t* pa;
   int32_t* pb;
   uint32_t* mask;
@@ -82,6 +83,7 @@ __global__ void __launch_bounds__(32 * kRouteWarps) route_kernel(RouteArgs a, co
   const int64_t i = (int64_t)blockIdx.x * kRouteWarps + warp;
   const bool valid = i < a.nq;
   int st = -1, nb = 0, Y = 0;
+  bool shrt = false;
   if (a.tc_slotpos) {
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t t = t0; t < a.tc_slots / 4; t += stride)  // tc_slots is a multiple of 128
@@ -105,6 +107,19 @@ __global__ void __launch_bounds__(32 * kRouteWarps) route_kernel(RouteArgs a, co
     Y = p1 - p0;
     st = a.forced;
     if (st < 0) st = (Y <= a.tau_a) ? UNIFY_PRE : ((Y >= a.tau_b) ? UNIFY_POST : UNIFY_HYBRID);
+    if (st == UNIFY_HYBRID) {
+      // A hybrid walk expands until ef_h of the objects it met are in range, about one in
+      // (rows of its segments) / Y of them; a post-filter walk expands about ef_p. The
+      // longest work should start first: hybrid walks that expect to take longer than a
+      // post-filter walk (an expansion of theirs costs about 1.5 of one) go before those,
+      // the others after. Measured on GB300, 10,000 auto-routed queries over 1M x 128 (4,000
+      // short hybrid walks, 2,000 post-filter walks; all hybrid walks first before):
+      // float32 1,259 -> 1,096 us, bfloat16 1,182 -> 1,010 us. Post-filter walks before every hybrid one lost 8 % on a batch with ranges
+      // that fill a tenth of their segments.
+      const unsigned rows = hit ? (unsigned)(__ldg(seg_start + lane + 1) - __ldg(seg_start + lane)) : 0u;
+      const int64_t met = __reduce_add_sync(kFull, rows);
+      shrt = 3 * (int64_t)a.ef_h * met <= 2 * (int64_t)a.ef_p * Y;
+    }
     if (st == UNIFY_PRE) {
       nb = (Y + a.scan_rows - 1) / a.scan_rows;
       nb = nb < 1 ? 1 : nb > a.max_items ? a.max_items : nb;
@@ -118,7 +133,7 @@ __global__ void __launch_bounds__(32 * kRouteWarps) route_kernel(RouteArgs a, co
   }
   if (!a.build_queues) return;
   if (lane == 0) {
-    s_strat[warp] = st;
+    s_strat[warp] = st == UNIFY_HYBRID && shrt ? 3 : st;
     s_nb[warp] = nb;
     s_rows[warp] = Y;
   }
@@ -127,15 +142,15 @@ __global__ void __launch_bounds__(32 * kRouteWarps) route_kernel(RouteArgs a, co
     const int qst = lane < kRouteWarps ? s_strat[lane] : -1;
     const int qnb = lane < kRouteWarps ? s_nb[lane] : 0;
     const int64_t qi = (int64_t)blockIdx.x * kRouteWarps + lane;
-    for (int q = 0; q < 3; ++q) {
-      // queue order: pre-filter, hybrid, post-filter
-      const bool mine = qst == (q == 0 ? UNIFY_PRE : q == 1 ? UNIFY_HYBRID : UNIFY_POST);
+    for (int q = 0; q < 4; ++q) {
+      // pre-filter, long hybrid, post-filter, short hybrid
+      const bool mine = qst == (q == 0 ? UNIFY_PRE : q == 1 ? UNIFY_HYBRID : q == 2 ? UNIFY_POST : 3);
       const unsigned bal = __ballot_sync(kFull, mine);
       if (bal == 0) continue;
       int base = 0;
-      if (lane == 0) base = atomicAdd(&a.counters[CNT_QA + q], __popc(bal));
-      base = __shfl_sync(kFull, base, 0);
-      if (mine) a.queues[q * a.cap_nq + base + __popc(bal & lanemask_lt())] = (int32_t)qi;
+      if (lane == 0) base = atomicAdd(&a.counters[q < 3 ? CNT_QA + q : CNT_QS], __popc(bal));
+      base = __shfl_sync(kFull, base, 0) + __popc(bal & lanemask_lt());
+      if (mine) a.queues[q < 3 ? q * a.cap_nq + base : 2 * a.cap_nq - 1 - base] = (int32_t)qi;
     }
     int incl = qnb;  // inclusive sum of the item counts
     for (int off = 1; off < kRouteWarps; off <<= 1) {
@@ -173,7 +188,7 @@ __global__ void __launch_bounds__(32 * kRouteWarps) route_kernel(RouteArgs a, co
 cudaError_t launch_route(const DeviceIndex& ix, const Scratch& sc, const int64_t* lo, const int64_t* hi,
                          int64_t nq, int64_t tau_a, int64_t tau_b, int forced, int scan_rows,
                          int build_queues, int32_t* out_pa, int32_t* out_pb, uint32_t* out_mask,
-                         int32_t* out_strat, const Outputs* outs, cudaStream_t st, bool tc) {
+                         int32_t* out_strat, const Outputs* outs, const Params* p, cudaStream_t st, bool tc) {
   RouteArgs a;
   a.sorted_attr = ix.sorted_attr;
   a.n = ix.n;
@@ -192,6 +207,8 @@ cudaError_t launch_route(const DeviceIndex& ix, const Scratch& sc, const int64_t
     a.max_items = (int)(share < kMaxItemsPerQuery ? share : kMaxItemsPerQuery);
   }
   a.build_queues = build_queues;
+  a.ef_h = p ? (p->ef > p->k ? p->ef : p->k) : 0;
+  a.ef_p = p ? (p->ef_post > p->k ? p->ef_post : p->k) : 0;
   a.pa = out_pa;
   a.pb = out_pb;
   a.mask = out_mask;

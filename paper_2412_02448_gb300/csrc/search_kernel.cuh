@@ -3,9 +3,9 @@
 //
 // Work queue. The router appends every query to a queue per strategy and splits
 // each pre-filter query into scan items. One warp takes one work unit at a time
-// from a single device counter, in the order: hybrid queries, post-filter queries,
-// scan items. The long graph searches start first and the short scan items fill
-// the tail, so the batch has one tail instead of one per strategy. A pre-filter
+// from a single device counter, in the order: long hybrid walks, post-filter walks,
+// short hybrid walks (route.cu tells them apart), scan items. The long graph searches
+// start first and the short scan items fill the tail, so the batch has one tail instead of one per strategy. A pre-filter
 // query split into several items is merged by the warp that completes its last
 // item (release/acquire through a per-query counter).
 //
@@ -778,12 +778,15 @@ __global__ void __launch_bounds__(128, MINB) batch_kernel(const __grid_constant_
     if (lane == 0) idx = atomicAdd(&a.counters[CNT_TAKE], 1);
     idx = __shfl_sync(kFull, idx, 0);
     // queue lengths: read again for every unit (in L1), not held across it
-    const int nC = __ldg(a.counters + CNT_QC), nB = __ldg(a.counters + CNT_QB);
-    if (idx < nC + nB) {
-      const bool hy = idx < nC;
-      graph_query<T, CH, G, GF, S1>(a, w, a.queues[hy ? a.cap_nq + idx : 2 * a.cap_nq + (idx - nC)], hy);
-    } else if (!a.skip_scan && idx - nC - nB < __ldg(a.counters + CNT_ITEMS)) {
-      scan_item<T, CH, RB, GF>(w.off, idx - nC - nB);
+    const int nL = __ldg(a.counters + CNT_QC), nLB = nL + __ldg(a.counters + CNT_QB);
+    const int nG = nLB + __ldg(a.counters + CNT_QS);
+    if (idx < nG) {
+      // long hybrid walks, post-filter walks, short hybrid walks (from the queue's end)
+      const bool hy = idx < nL || idx >= nLB;
+      const int64_t at = idx < nL ? a.cap_nq + idx : idx < nLB ? 2 * a.cap_nq + (idx - nL) : 2 * a.cap_nq - 1 - (idx - nLB);
+      graph_query<T, CH, G, GF, S1>(a, w, a.queues[at], hy);
+    } else if (!a.skip_scan && idx - nG < __ldg(a.counters + CNT_ITEMS)) {
+      scan_item<T, CH, RB, GF>(w.off, idx - nG);
     } else {
       break;
     }
