@@ -259,8 +259,6 @@ __device__ __forceinline__ int select_s1(const BatchArgs& a, const WarpMem& w, i
   const int32_t* adj = (l == 0 ? a.adj0 : a.adjU) + row * (a.S * a.M);
   const unsigned char* orow = a.vt + (int64_t)o * a.row_bytes;
   const float sc = a.scale ? __ldg(a.scale + o) : 1.f;
-  // narrow rows: all 32 of a batch in flight
-  constexpr int GS = CH == 1 && T::kRawRegs == 1 ? 32 : G;
   __syncwarp();
   float4* const xo = reinterpret_cast<float4*>(w.at(w.xo()));
   for (int c = lane; c < a.dp4; c += 32) xo[c] = value4<T>(T::load(orow, c, sc), sc);
@@ -278,7 +276,7 @@ __device__ __forceinline__ int select_s1(const BatchArgs& a, const WarpMem& w, i
   for (int b0 = 0; b0 < tot; b0 += 32) {
     const int cid = next;
     next = neighbour(b0 + 32 + lane);
-    const float dv = batch_dist<T, CH, GS>(w.xo(), cid, a.vt, a.row_bytes, a.scale, a.dp4, scratch);
+    const float dv = batch_dist<T, CH, G, CH == 1 && T::kRawRegs == 1>(w.xo(), cid, a.vt, a.row_bytes, a.scale, a.dp4, scratch);
     ns = topk_offer(selk, ns, a.m < 64 ? a.m : 64, cid >= 0 ? make_key(dv, cid) : kKeyMax, w.SK());
   }
   for (int t = lane; t < ns; t += 32) sts32(w.nadj(0) + 4 * t, key_id(lds64(selk + 8 * t)));
