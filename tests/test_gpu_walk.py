@@ -26,7 +26,7 @@ def _table(d):
     return x.astype(np.float32), attr, q.astype(np.float32), lo, lo + w - 1
 
 
-@pytest.fixture(scope="module", params=[3, 17, 32, 100, 129, 200, 515])
+@pytest.fixture(scope="module", params=[3, 17, 32, 100, 129, 200, 300, 515])
 def table(request, tmp_path_factory):
     import hsig_build
     import oracle
@@ -80,3 +80,31 @@ def test_scan_items_equal_exact(table, nq, k, scan_rows):
                           params=U.Params.defaults(scan_rows=scan_rows, dtype=dtype)))
         np.testing.assert_array_equal(r["ids"], ids)
         np.testing.assert_array_equal(r["count"], cnt)
+
+
+@pytest.mark.parametrize("d", [17, 96, 128, 300, 600])
+def test_narrow_rows_equal_oracle(d, tmp_path):
+    """BF16 and FP8 storage on vectors that both hold exactly (integers 0..7, every vector's
+    largest coordinate 7: the FP8 scale is 1/64 and every code exact), both selections: the
+    rows of float32 storage, which are the oracle's."""
+    import hsig_build
+    import oracle
+    import paper_2412_02448_gb300 as U
+    x, attr, q, lo, hi = _table(d)
+    top = float(max(x.max(), q.max(), 1.0))
+    x, q = np.rint(x * (7.0 / top)), np.rint(q * (7.0 / top))
+    x[np.arange(N), np.arange(N) % d] = 7.0
+    x, q = x.astype(np.float32), q.astype(np.float32)
+    path = str(tmp_path / "t.idx")
+    hsig_build.build_index(x, attr, path, S, M, 40, seed=5)
+    ix, oi = U.Index(path, device=0), oracle.OracleIndex(path)
+    for strategy, sel, m in (("hybrid", 2, 48), ("hybrid", 1, 40), ("post", 2, 16), ("pre", 2, 16)):
+        o = oi.search(q, lo, hi, 10, ef=64, ef_post=64, m=m, strategy=strategy, selection=sel)
+        for dtype in (U.FP32, U.BF16, U.FP8E4M3):
+            p = U.Params.defaults(ef=64, ef_post=64, m=m, selection=sel, dtype=dtype, cand_cap=4096)
+            r = _np(ix.search(q, lo, hi, 10, strategy=strategy, params=p))
+            assert not r["status"].any()
+            np.testing.assert_array_equal(r["ids"], o["ids"], err_msg=f"{strategy} S{sel} dtype {dtype}")
+            np.testing.assert_array_equal(r["count"], o["count"])
+    ix.close()
+    oi.close()
