@@ -13,7 +13,7 @@ namespace unify {
 // warps for longer than a 4 MB item takes, so that finer items only take issue slots from
 // them (2 % slower at 1,003 queries): there a batch counts sixteenfold.
 // Measured on GB300 against items of 8,192 rows: 17 queries over 15,000 rows of 512 B
-// each 585 -> 63 us; 301 queries over 4,200 rows of 3,840 B 4,900 -> 928 us.
+// each 585 -> 63 us; 301 queries over 4,200 rows of 3,840 B 4,900 -> 985 us.
 int scan_item_rows(const DeviceIndex& ix, const Params& p, int64_t nq, int strategy) {
   const int64_t row_bytes = (int64_t)ix.dp * 4;  // a row's arithmetic is the same in every storage format
   const int64_t slots = 16ll * ix.num_sms;

@@ -57,7 +57,7 @@
 // computes 32 rows per step, eight lanes per row (4 shuffles per 16 rows instead of 16,
 // all loads of a batch in flight); keys beating the current k-th are inserted into a
 // sorted top-k. Bound by HBM once a batch fills the device: 301 queries over 4,150 rows of
-// 3,840 B each run at 5.2 TB/s of gathered rows (928 us).
+// 3,840 B each run at 4.9 TB/s of gathered rows (985 us).
 //
 // Bounds (checked by reading, against the buffers the launch receives):
 // E[< cand_cap], ann[< ann_cap], vis[< 2^vis_log2], clist[< 32], SK[< 32], nadj and
