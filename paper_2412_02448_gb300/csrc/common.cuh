@@ -86,7 +86,7 @@ __device__ __forceinline__ int warp_lower_bound(saddr a, int n, uint64_t x, unsi
   const int lane = lane_id();
   const int step = (n + 31) >> 5;
   const int li = (lane + 1) * step - 1;
-  const uint64_t sample = li < n ? lds64(a + 8 * li) : kKeyMax;
+  const uint64_t sample = (unsigned)li < (unsigned)n ? lds64(a + 8 * li) : kKeyMax;  // li is -1 where n = 0
   int rank = 0;
 #pragma unroll 1
   for (unsigned rest = kb; rest; rest &= rest - 1) {
