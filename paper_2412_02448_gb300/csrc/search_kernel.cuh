@@ -561,6 +561,7 @@ __device__ __forceinline__ void graph_query(const BatchArgs& a, const WarpMem& w
       nA = search_layer<T, CH, G, S1>(a, w, hy, l == 0, l > 0 ? 1 : cold->efl0, ep_key, ep_in);
       if (l > 0 && nA > 0) ep_key = lds64(w.ann()) & ~1ull;
       l = cold->l;
+      __syncwarp();  // lane 0 stores the next layer's number only after every lane has read this one's
     }
     qi = cold->qi;
     if (a.rerank > 0) {
