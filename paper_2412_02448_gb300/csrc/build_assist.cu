@@ -197,6 +197,8 @@ __device__ int build_search(const BuildArgs& a, const BuildWarp& w, int l, int j
       if (w.vis[h] == cid) cid = -1;
       else w.vis[h] = cid;
     }
+    // a chunk that a caller handed over may repeat an id: its first place counts
+    if ((__match_any_sync(kFull, cid >= 0 ? cid : ~lane) & lanemask_lt()) != 0) cid = -1;
     __syncwarp();
     const unsigned vm = __ballot_sync(kFull, cid >= 0);
     const int nc = __popc(vm);
@@ -362,7 +364,9 @@ __global__ void __launch_bounds__(32 * kBuildWarps, 4) reverse_kernel(RevArgs a)
   const int M = a.M;
   int c = a.cnt[ch];
   const uint64_t key = lane < c ? make_key(a.adjd[ch * M + lane], a.adj[ch * M + lane]) : kKeyMax;
-  const int at = rank_plain(key, __ballot_sync(kFull, lane < c), sa(sSK[warp]));
+  const unsigned held = __ballot_sync(kFull, lane < c);
+  const int at = rank_plain(key, held, sa(sSK[warp])) +
+                 __popc(__match_any_sync(kFull, (unsigned long long)key) & held & lanemask_lt());  // equal keys: a place each
   if (lane < c) K[at] = key;
   __syncwarp();
   const int64_t e1 = a.g_start[g + 1];

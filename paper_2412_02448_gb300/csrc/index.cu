@@ -183,6 +183,23 @@ __global__ void marked_kernel(const int32_t* __restrict__ adj, const uint32_t* _
   }
 }
 
+// Sets *out where a chunk names a neighbour twice, or one that does not belong to the
+// chunk's segment: a file without either names every neighbour of a row once. The builder's
+// files are such; searches of any other look for repetitions as they go (2 to 4 % slower on
+// GB300, which is why they do not in general).
+__global__ void repeats_kernel(const int32_t* __restrict__ adj, int64_t chunks, int S, int M,
+                               const int32_t* __restrict__ pos, const int32_t* __restrict__ seg_start, int* out) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < chunks * M; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t ch = i / M;
+    const int32_t v = adj[i];
+    if (v < 0) continue;
+    const int j = (int)(ch % S), p = pos[v];
+    bool bad = p < seg_start[j] || p >= seg_start[j + 1];
+    for (int64_t e = ch * M; e < i; ++e) bad |= adj[e] == v;
+    if (bad) *out = 1;
+  }
+}
+
 void free_device(DeviceIndex& ix) {
   void* ptrs[] = {ix.vec, ix.vec_sorted, ix.sorted_ids, ix.sorted_attr, ix.pos, ix.upper_base, ix.adj0,
                   ix.gadj0, ix.adjU, ix.gadjU, ix.seg_bounds, ix.seg_start, ix.vt_bf16, ix.vts_bf16,
@@ -420,7 +437,17 @@ extern "C" int unify_load_index(const char* path, int device, unify_index_t** ou
                                ix.xn_bf16_sorted, ix.xn_f32_sorted, ix.xn_fp8_sorted);
     e = cudaGetLastError();
   }
+  int* d_rep = nullptr;
+  if (e == cudaSuccess) e = cudaMalloc(&d_rep, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(d_rep, 0, sizeof(int));
+  for (int part = 0; part < 2 && e == cudaSuccess; ++part) {
+    const int64_t rows = part == 0 ? ix.n : ix.n_upper;  // validated rows
+    repeats_kernel<<<1024, 256>>>(part == 0 ? ix.adj0 : ix.adjU, rows * ix.S, ix.S, ix.M, ix.pos, ix.seg_start, d_rep);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(&ix.repeats, d_rep, sizeof(int), cudaMemcpyDeviceToHost);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  if (d_rep) cudaFree(d_rep);
   if (d_attr) cudaFree(d_attr);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ix.num_sms, cudaDevAttrMultiProcessorCount, device);
   if (e != cudaSuccess) {

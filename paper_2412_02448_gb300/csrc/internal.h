@@ -37,6 +37,7 @@ struct DeviceIndex {
   int32_t* upper_base = nullptr;
   int32_t* adj0 = nullptr;      // (n, S, M), -1 padded
   int32_t* adjU = nullptr;      // (n_upper, S, M)
+  int repeats = 0;              // a row may name a neighbour more than once (see repeats_kernel)
   // bitmap-marked neighbours, compacted in slot order (-1 past the end): the first GW
   // marked slots of every row
   int GW = 0;                   // the largest number of marked slots of a row, at most 64, rounded up to 4

@@ -80,6 +80,7 @@ cudaError_t launch_batch(const DeviceIndex& ix, const Scratch& sc, const float* 
   a.adjU = ix.adjU;
   a.gadjU = ix.gadjU;
   a.GW = ix.GW;
+  a.repeats = ix.repeats;
   a.upper_base = ix.upper_base;
   a.pos = ix.pos;
   a.seg_start = ix.seg_start;

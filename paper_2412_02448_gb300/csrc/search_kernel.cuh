@@ -63,8 +63,10 @@
 // E[< cand_cap], ann[< ann_cap], vis[< 2^vis_log2], clist[< 32], SK[< 32], nadj and
 // table[< kSlotTable]; S1 keeps its 64 keys in nadj(1) and the table's first 32 ints, its
 // list of 32 ids after them; ids come from validated adjacency
-// (0 <= id < n < 2^30); upper-layer rows exist for every object reached on that layer
-// (validated levels); scan rows lie in [pa, pb) and loads clamp to the last valid row.
+// (0 <= id < n < 2^30), and where a row repeats one only its first place is inserted
+// (sorted_insert keeps positions apart by distinct keys); upper-layer rows exist for every
+// object reached on that layer (validated levels); scan rows lie in [pa, pb) and loads
+// clamp to the last valid row.
 #pragma once
 
 #include "common.cuh"
@@ -106,6 +108,7 @@ struct BatchArgs {
   int32_t* counters;
   int k, ef_h, ef_p, m, cand_cap, ann_cap, vis_log2, max_exp;
   Conj cj;  // second-attribute predicate (attr2 == nullptr: none)
+  int repeats;  // a row of the file may name a neighbour more than once
   int s1;  // hybrid selection S1 (the m neighbours nearest to the expanded object) instead of S2
   int warp_bytes, off_q, off_E, off_ann;
   int skip_scan;  // the pre-filter queries were searched by the tensor-core scan
@@ -277,7 +280,7 @@ __device__ __forceinline__ int select_s1(const BatchArgs& a, const WarpMem& w, i
     const int cid = next;
     next = neighbour(b0 + 32 + lane);
     const float dv = batch_dist<T, CH, G, CH == 1 && T::kRawRegs == 1>(w.xo(), cid, a.vt, a.row_bytes, a.scale, a.dp4, scratch);
-    ns = topk_offer(selk, ns, a.m < 64 ? a.m : 64, cid >= 0 ? make_key(dv, cid) : kKeyMax, w.SK());
+    ns = topk_offer(selk, ns, a.m < 64 ? a.m : 64, cid >= 0 ? make_key(dv, cid) : kKeyMax, w.SK(), a.repeats != 0);
   }
   for (int t = lane; t < ns; t += 32) sts32(w.nadj(0) + 4 * t, key_id(lds64(selk + 8 * t)));
   __syncwarp();
@@ -433,6 +436,11 @@ __device__ __forceinline__ int search_layer(const BatchArgs& a, WarpMem w, bool 
         }
         const int c = lane < m ? (int)lds32(list + 4 * (c0 + lane)) : 0;
         const int id = c & kIdMask;
+        // where a row of the file may name a neighbour twice, its first place counts
+        // (sorted_insert wants distinct keys)
+        unsigned cand = m < 32 ? (1u << m) - 1u : kFull;
+        if (a.repeats)
+          cand &= __ballot_sync(kFull, (__match_any_sync(kFull, lane < m ? id : ~lane) & lanemask_lt()) == 0);
         const int pv = hy && c < 0 ? __ldg(a.pos + id) : 0;
         const bool two = hy && base && a.cj.attr2 != nullptr;
         const int64_t v2 = two && lane < m ? __ldg(a.cj.attr2 + id) : 0;
@@ -449,7 +457,7 @@ __device__ __forceinline__ int search_layer(const BatchArgs& a, WarpMem w, bool 
         }
         const uint64_t key = graph_key(dist, id);
         const saddr last = w.ann() + 8 * (efl - 1);  // for post, E is w.ann
-        unsigned kb = __ballot_sync(kFull, lane < m && key < (nA >= efl ? lds64(last) & ~1ull : kKeyMax));
+        unsigned kb = cand & __ballot_sync(kFull, key < (nA >= efl ? lds64(last) & ~1ull : kKeyMax));
         if (kb == 0) continue;
         // where E might overflow: block by block, each against the ann of its own start
         unsigned ends = 0;
@@ -463,7 +471,7 @@ __device__ __forceinline__ int search_layer(const BatchArgs& a, WarpMem w, bool 
           if (hy && ends) {
             const int b1 = __ffs(ends);
             ends &= ends - 1;
-            kb = __ballot_sync(kFull, lane >= b0 && lane < b1 && key < (nA >= efl ? lds64(last) : kKeyMax));
+            kb = cand & __ballot_sync(kFull, lane >= b0 && lane < b1 && key < (nA >= efl ? lds64(last) : kKeyMax));
             b0 = b1;
           }
           if (kb) insert_batch(a, w, hy, efl, key, inr, kb, nE, nA, cursor, truncated);

@@ -346,13 +346,15 @@ __device__ __forceinline__ int rank_plain(uint64_t key, unsigned kb, saddr SK) {
 }
 
 // Keeps the k smallest keys: inserts the lanes' keys (plain (distance, id) keys) that
-// beat the current k-th into topk[0, nt). SK as in rank_among.
-__device__ __forceinline__ int topk_offer(saddr topk, int nt, int k, uint64_t key, saddr SK) {
+// beat the current k-th into topk[0, nt). SK as in rank_among. The keys of one call are
+// distinct, or twins is set: equal ones then take a place each, in the lanes' order.
+__device__ __forceinline__ int topk_offer(saddr topk, int nt, int k, uint64_t key, saddr SK, bool twins = false) {
   const uint64_t thr = (nt >= k) ? lds64(topk + 8 * (k - 1)) : kKeyMax;
   const bool pass = key < thr;
   const unsigned bal = __ballot_sync(kFull, pass);
   if (bal == 0) return nt;
-  const int less = rank_plain(key, bal, SK);
+  int less = rank_plain(key, bal, SK);
+  if (twins) less += __popc(__match_any_sync(kFull, (unsigned long long)key) & bal & lanemask_lt());
   const int rank = warp_rank(topk, nt, key, bal);
   return sorted_insert(topk, nt, k, key, rank, less, bal);
 }

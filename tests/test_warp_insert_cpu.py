@@ -72,6 +72,9 @@ static unsigned __reduce_or_sync(unsigned, unsigned v) {
 static unsigned __reduce_min_sync(unsigned, unsigned v) {
   return all<unsigned>(v, [] { unsigned b = ~0u; for (int i = 0; i < 32; ++i) b = std::min(b, x32(i)); return b; });
 }
+static unsigned __match_any_sync(unsigned, unsigned long long v) {
+  return all<uint64_t>(v, [v] { unsigned b = 0; for (int i = 0; i < 32; ++i) b |= (unsigned)(g_x[i] == v) << i; return b; });
+}
 static uint64_t __shfl_sync(unsigned, uint64_t v, int src) {
   return all<uint64_t>(v, [src] { return g_x[src & 31]; });
 }
@@ -86,16 +89,16 @@ template <class F> static void warp(F f) {
   for (int i = 0; i < 32; ++i) t.emplace_back([&f, i] { t_lane = i; f(i); });
   for (auto& x : t) x.join();
 }
-// Offers `rounds` x 32 keys to a list of k; returns its length (list in out), or -1 after
+// Offers `rounds` x 32 keys to a list of k (twins: equal keys among those of a round); returns its length (list in out), or -1 after
 // an access outside the arrays. One array entry beyond the list may not be read.
-extern "C" int offer(const uint64_t* keys, int rounds, int k, uint64_t* out) {
+extern "C" int offer(const uint64_t* keys, int rounds, int k, int twins, uint64_t* out) {
   g_faults = 0;
   std::fill(g_arr, g_arr + kRoom, 0x5555555555555555ull);
   int n = 0;
   for (int r = 0; r < rounds; ++r) {
     int nn[32];
     g_len = std::max(k, n);
-    warp([&](int i) { nn[i] = topk_offer(kArr, n, k, keys[32 * r + i], kSK); });
+    warp([&](int i) {nn[i] = topk_offer(kArr, n, k, keys[32 * r + i], kSK, twins != 0); });
     n = nn[0];
   }
   std::copy(g_arr, g_arr + n, out);
@@ -138,7 +141,7 @@ def lib(tmp_path_factory):
     so = str(d / "w.so")
     subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-pthread", str(src), "-o", so], check=True)
     lib = ctypes.CDLL(so)
-    lib.offer.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_void_p]
+    lib.offer.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_void_p]
     lib.ranks.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_uint]
     return lib
 
@@ -164,7 +167,20 @@ def test_topk_offer(lib, k, lanes):
     keys = np.full((rounds, 32), np.iinfo(np.uint64).max, np.uint64)
     keys[:, :lanes] = rng.choice(1 << 20, size=rounds * lanes, replace=False).reshape(rounds, lanes)
     out = np.zeros(600, np.uint64)
-    n = lib.offer(keys.ctypes.data, rounds, k, out.ctypes.data)
+    n = lib.offer(keys.ctypes.data, rounds, k, 0, out.ctypes.data)
     want = np.sort(keys[:, :lanes].ravel())[:k]
+    assert n == len(want)
+    np.testing.assert_array_equal(out[:n], want)
+
+
+@pytest.mark.parametrize("k", [1, 7, 40, 256])
+def test_topk_offer_twins(lib, k):
+    """Offers that repeat keys, within themselves and of earlier ones: the k smallest of the
+    multiset, every position of the list written."""
+    rng = np.random.default_rng([k, 9])
+    keys = rng.integers(0, 60, (12, 32)).astype(np.uint64)
+    out = np.zeros(600, np.uint64)
+    n = lib.offer(keys.ctypes.data, 12, k, 1, out.ctypes.data)
+    want = np.sort(keys.ravel())[:k]
     assert n == len(want)
     np.testing.assert_array_equal(out[:n], want)
