@@ -531,7 +531,7 @@ __device__ __forceinline__ void graph_query(const BatchArgs& a, const WarpMem& w
       cold->per = per;
       cold->slots = !hy ? a.GW : S1 ? Sp : Sp * per;  // S1: select_s1 takes the number of segments
       cold->efl0 = hy ? (a.ef_h > a.k ? a.ef_h : a.k) : (a.ef_p > a.k ? a.ef_p : a.k);
-      cold->n_dist = 1;
+      cold->n_dist = 0;
       cold->n_exp = 0;
       cold->status = 0;
       cold->mask = mask;
@@ -550,6 +550,7 @@ __device__ __forceinline__ void graph_query(const BatchArgs& a, const WarpMem& w
     const float d0 = batch_dist<T, CH, G>(w.q(), lane == 0 ? a.entry_global : -1, a.vt, a.row_bytes, a.scale, a.dp4,
                                           w.clist());
     uint64_t ep_key = graph_key(__shfl_sync(kFull, d0, 0), a.entry_global);
+    if (lane == 0) cold->n_dist = 1;
     int nA = 0;
 #pragma unroll 1
     for (int l = a.max_level; l >= 0; --l) {
@@ -628,7 +629,7 @@ __device__ __forceinline__ void graph_query(const BatchArgs& a, const WarpMem& w
     a.o.count[qi] = cnt;
     if (a.o.status) a.o.status[qi] = cold->status;
     if (a.o.counters) {
-      a.o.counters[4 * (int64_t)qi] = cold->mask == 0 && hy ? 0 : cold->n_dist;
+      a.o.counters[4 * (int64_t)qi] = cold->n_dist;
       a.o.counters[4 * (int64_t)qi + 1] = cold->n_exp;
       a.o.counters[4 * (int64_t)qi + 2] = cold->t_start;
       a.o.counters[4 * (int64_t)qi + 3] = us_since_start(a.counters);
