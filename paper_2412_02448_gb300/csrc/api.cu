@@ -318,7 +318,7 @@ int run_search(unify_index_t* idx, const float* q, const int64_t* lo, const int6
   if (!(tc && strategy == UNIFY_PRE)) {
     NvtxRange r("unify:search kernel");
     PhaseTimer t(idx->tm, 1, st);
-    e = launch_batch(idx->ix, sc, q, p, o, st, tc, cj);
+    e = launch_batch(idx->ix, sc, q, p, o, st, tc, cj, strategy == UNIFY_PRE);
   }
   if (e != cudaSuccess) return cuda_fail(e, "search kernel");
   return UNIFY_OK;

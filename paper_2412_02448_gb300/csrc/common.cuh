@@ -155,25 +155,39 @@ __device__ __forceinline__ float oct_transpose_reduce(float (&v)[V]) {
 //
 // Raw is a chunk as loaded (16, 8 or 4 bytes: 4, 2 or 1 registers); decode() turns it
 // into four floats, at use.
-// Read-only loads that leave no line in L1: a row is read once by its warp, and the L1
-// beside a full shared memory is small. Volatile: all loads of a group stay together in
+// Read-only loads that leave no line in L1 (kL1: that do): a row is read once by its warp,
+// and the L1 beside a full shared memory is small. Volatile: all loads of a group stay together in
 // front of the arithmetic. Otherwise the compiler moves each into the branch that uses
 // its chunk, and a group costs four memory latencies instead of one.
+template <bool kL1>
 __device__ __forceinline__ float4 load_stream16(const void* p) {
   float4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
-      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-      : "l"(p));
+  if constexpr (kL1)
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+        : "l"(p));
+  else
+    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+        : "l"(p));
   return v;
 }
+template <bool kL1>
 __device__ __forceinline__ uint2 load_stream8(const void* p) {
   uint2 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  if constexpr (kL1)
+    asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  else
+    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
   return v;
 }
+template <bool kL1>
 __device__ __forceinline__ uint32_t load_stream4(const void* p) {
   uint32_t v;
-  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  if constexpr (kL1)
+    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  else
+    asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
 }
 
@@ -182,8 +196,9 @@ struct StoreF32 {
   static constexpr bool kScaled = false;
   using Raw = float4;
   static constexpr int kRawRegs = 4;
+  template <bool kL1 = false>
   __device__ static __forceinline__ Raw load_raw(const unsigned char* row, int c) {
-    return load_stream16(row + 16 * c);
+    return load_stream16<kL1>(row + 16 * c);
   }
   __device__ static __forceinline__ Raw zero_raw() { return make_float4(0.f, 0.f, 0.f, 0.f); }
   __device__ static __forceinline__ float4 decode(const Raw& r) { return r; }
@@ -194,8 +209,9 @@ struct StoreBF16 {  // bfloat16, converted from float32 with round-to-nearest-ev
   static constexpr bool kScaled = false;
   using Raw = uint2;
   static constexpr int kRawRegs = 2;
+  template <bool kL1 = false>
   __device__ static __forceinline__ Raw load_raw(const unsigned char* row, int c) {
-    return load_stream8(row + 8 * c);
+    return load_stream8<kL1>(row + 8 * c);
   }
   __device__ static __forceinline__ Raw zero_raw() { return make_uint2(0u, 0u); }
   __device__ static __forceinline__ float4 decode(const Raw& u) {
@@ -215,8 +231,9 @@ struct StoreFP8 {
   static constexpr bool kScaled = true;
   using Raw = uint32_t;
   static constexpr int kRawRegs = 1;
+  template <bool kL1 = false>
   __device__ static __forceinline__ Raw load_raw(const unsigned char* row, int c) {
-    return load_stream4(row + 4 * c);
+    return load_stream4<kL1>(row + 4 * c);
   }
   __device__ static __forceinline__ Raw zero_raw() { return 0u; }
   __device__ static __forceinline__ float4 decode(const Raw& u) {

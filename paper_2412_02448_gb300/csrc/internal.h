@@ -160,7 +160,8 @@ cudaError_t launch_route(const DeviceIndex& ix, const Scratch& sc, const int64_t
                          int build_queues, int32_t* out_pa, int32_t* out_pb, uint32_t* out_mask,
                          int32_t* out_strat, const Outputs* outs, const Params* p, cudaStream_t st, bool tc = false);
 cudaError_t launch_batch(const DeviceIndex& ix, const Scratch& sc, const float* q, const Params& p,
-                         const Outputs& o, cudaStream_t st, bool skip_scan = false, const Conj* cj = nullptr);
+                         const Outputs& o, cudaStream_t st, bool skip_scan = false, const Conj* cj = nullptr,
+                         bool scan_only = false);  // scan_only: every query is a pre-filter query
 bool tc_scan_available(const DeviceIndex& ix, const Params& p);
 size_t tc_query_row_bytes(int d);  // bytes of one query row of the tensor-core scan, any format
 cudaError_t launch_tcscan(const DeviceIndex& ix, const Scratch& sc, const float* q, int64_t nq, const Params& p,

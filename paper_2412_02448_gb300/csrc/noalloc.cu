@@ -130,7 +130,7 @@ extern "C" int unify_search_noalloc(unify_index_t* idx, const float* q, const in
                    scan_item_rows(idx->ix, prm, nq, st_code), 1, sc.pa, sc.pb,
                    sc.mask, sc.strat, &o, &prm, st);
   if (e != cudaSuccess) return cuda_fail(e, "route kernel");
-  e = launch_batch(idx->ix, sc, q, prm, o, st);
+  e = launch_batch(idx->ix, sc, q, prm, o, st, false, nullptr, st_code == UNIFY_PRE);
   if (e != cudaSuccess) return cuda_fail(e, "search kernel");
   return UNIFY_OK;
 }

@@ -7,19 +7,24 @@ namespace unify {
 // Rows per scan work item, at most p.scan_rows. An item is one warp's, so it is the
 // granularity of the batch's tail and, when there are few queries, all the parallelism
 // there is: with fewer queries than resident warps (16 per SM) it shrinks in proportion,
-// from 1 MB of float32 rows down to 64 KB, and it grows with the batch up to 4 MB; never
-// below 64 rows, nor below 4 rows per key kept (each item sorts its own list of the kept
-// keys, which the query's last item merges). In a routed batch the graph walks hold most
-// warps for longer than a 4 MB item takes, so that finer items only take issue slots from
-// them (2 % slower at 1,003 queries): there a batch counts sixteenfold.
+// from 1 MB of float32 rows down to 64 KB, and it grows with a pre-filter batch up to 4 MB;
+// never below 64 rows, nor below 4 rows per key kept (each item sorts its own list of the
+// kept keys, which the query's last item merges). In a routed batch the graph walks hold most
+// warps for longer than an item takes, and finer items only take issue slots from them (2 %
+// slower at 1,003 queries with 64 KB): there a batch counts sixteenfold, up to 512 KB, beyond
+// which the items after the walks are too few for an even end: 5,000 log-uniform queries
+// over 1M x 128 at the tuned parameters 2,091 us with 4 MB, 1,863 with 1 MB, 1,878 with 512
+// KB, 2,042 with 64 KB; 10,000 queries of five widths 2,065, 1,970, 1,974 and 2,095; 5,000
+// of these 1,119, 1,062, 1,023 and 1,083.
 // Measured on GB300 against items of 8,192 rows: 17 queries over 15,000 rows of 512 B
-// each 585 -> 63 us; 301 queries over 4,200 rows of 3,840 B 4,900 -> 985 us.
+// each 585 -> 50 us; 301 queries over 4,200 rows of 3,840 B 4,900 -> 609 us.
 int scan_item_rows(const DeviceIndex& ix, const Params& p, int64_t nq, int strategy) {
   const int64_t row_bytes = (int64_t)ix.dp * 4;  // a row's arithmetic is the same in every storage format
   const int64_t slots = 16ll * ix.num_sms;
   int64_t bytes = (1ll << 20) * (strategy == UNIFY_AUTO ? 16 : 1) * nq / slots;
   if (bytes < (64 << 10)) bytes = 64 << 10;
-  if (bytes > (4 << 20)) bytes = 4 << 20;
+  const int64_t most = strategy == UNIFY_AUTO ? 512 << 10 : 4 << 20;
+  if (bytes > most) bytes = most;
   const int64_t kept = rerank_count(p) > p.k ? rerank_count(p) : p.k;
   int64_t rows = bytes / row_bytes;
   if (rows < 64) rows = 64;
@@ -45,7 +50,7 @@ int batch_smem_per_warp(const Params& p) {
 }
 
 cudaError_t launch_batch(const DeviceIndex& ix, const Scratch& sc, const float* q, const Params& p,
-                         const Outputs& o, cudaStream_t st, bool skip_scan, const Conj* cj) {
+                         const Outputs& o, cudaStream_t st, bool skip_scan, const Conj* cj, bool scan_only) {
   BatchArgs a;
   a.cj = cj ? *cj : Conj{};
   a.skip_scan = skip_scan ? 1 : 0;
@@ -105,6 +110,14 @@ cudaError_t launch_batch(const DeviceIndex& ix, const Scratch& sc, const float* 
   a.ann_cap = batch_ann_cap(p);
   a.vis_log2 = p.vis_log2;
   a.max_exp = p.max_exp;
+  if (scan_only) {
+    // Nothing walks: no visited filter, the lists alone. With the default parameters 16 warps
+    // per SM instead of the 12 that fit beside the walks' buffers (the 128-register build):
+    // 4,000 queries over 1M x 128 BF16 1,300 -> 955 us, float32 1,552 -> 1,346.
+    a.cand_cap = p.k;
+    a.ann_cap = p.k > a.rerank ? p.k : a.rerank;
+    a.vis_log2 = 6;
+  }
   layout(a);
   a.o = o;
   const int fit = (227 * 1024 - kArgsBytes) / a.warp_bytes;

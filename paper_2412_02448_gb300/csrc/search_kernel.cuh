@@ -662,7 +662,7 @@ static __device__ __noinline__ int merge_lists(saddr off, const uint64_t* lists,
   return nt;
 }
 
-template <class T, int CH, int RB, int GF>
+template <class T, int CH, int RB, int GF, bool kL1>
 __device__ __noinline__ void scan_item(uint32_t off, int it) {
   const BatchArgs& a = shared_args();
   const WarpMem w{off, a};
@@ -679,8 +679,16 @@ __device__ __noinline__ void scan_item(uint32_t off, int it) {
   const int r1 = min(pb, r0 + rpb);
   const int64_t l2 = a.cj.attr2 ? a.cj.lo2[qi] : 0, h2 = a.cj.attr2 ? a.cj.hi2[qi] : 0;
   load_query(reinterpret_cast<float4*>(w.at(w.q())), a.q + (int64_t)qi * a.d, a.d, a.dp4);
-  // eight lanes per row (as group_dist): row base + 4 r + g, r < 8, is lanes 8 g .. 8 g + 7's;
-  // RB of the eight steps r load together
+  // Eight lanes per row (as group_dist): row base + 4 r + g, r < 8, is lanes 8 g .. 8 g + 7's;
+  // RB of the eight steps r load together, 32 chunks of each row at a time. The arguments are
+  // copied out of shared memory first: every insertion would make them be read again. The
+  // loop over a row's chunk blocks stays a loop: unrolled, the row loads of all blocks crowd
+  // the registers (1.1 KB of spills at 960 elements, 90 bytes so).
+  const int dp4 = a.dp4, row_bytes = a.row_bytes;
+  const unsigned char* const rows = a.vts;
+  const float* const row_scale = a.scale_sorted;
+  const int32_t* const sorted_ids = a.sorted_ids;
+  const saddr qs = w.q();
   const int j = lane & 7, g = lane >> 3;
   int nt = 0;
 #pragma unroll 1
@@ -694,30 +702,28 @@ __device__ __noinline__ void scan_item(uint32_t off, int it) {
 #pragma unroll
       for (int r = 0; r < RB; ++r) {
         const int row = min(base + 4 * (h + r) + g, r1 - 1);
-        src[r] = a.vts + (int64_t)row * a.row_bytes;
-        sc[r] = T::kScaled ? __ldg(a.scale_sorted + row) : 1.f;
+        src[r] = rows + (int64_t)row * row_bytes;
+        sc[r] = T::kScaled ? __ldg(row_scale + row) : 1.f;
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[r][i] = 0.f;
       }
-#pragma unroll
-      for (int t = 0; t < CH; ++t) {
+#pragma unroll 1
+      for (int c0 = 0; CH == 1 ? c0 < 1 : c0 < dp4; c0 += 32) {
         Held<T> x[RB][4];
 #pragma unroll
         for (int r = 0; r < RB; ++r)
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const int c = 32 * t + 8 * i + j;
-            x[r][i] = c < a.dp4 ? T::load_raw(src[r], c) : T::zero_raw();
+            const int c = c0 + 8 * i + j;
+            x[r][i] = c < dp4 ? T::template load_raw<kL1>(src[r], c) : T::zero_raw();
           }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const int c = 32 * t + 8 * i + j;
-          if (c < a.dp4) {
-            const float4 q = lds_f4(w.q() + 16 * c);
+          const int c = c0 + 8 * i + j;
+          if (c < dp4) {
+            const float4 q = lds_f4(qs + 16 * c);
 #pragma unroll
-            for (int r = 0; r < RB; ++r) {
-              acc[r][i] = sum_sq<T>(q, T::decode(x[r][i]), sc[r], acc[r][i]);
-            }
+            for (int r = 0; r < RB; ++r) acc[r][i] = sum_sq<T>(q, T::decode(x[r][i]), sc[r], acc[r][i]);
           }
         }
       }
@@ -728,7 +734,7 @@ __device__ __noinline__ void scan_item(uint32_t off, int it) {
     const int row = base + 4 * j + g;
     uint64_t key = kKeyMax;
     if (row < r1) {
-      const int32_t id = __ldg(a.sorted_ids + row);
+      const int32_t id = __ldg(sorted_ids + row);
       if (conj_ok(a, id, l2, h2)) key = make_key(dist, id);
     }
     nt = topk_offer(topk, nt, kk, key, w.SK());
@@ -775,6 +781,11 @@ __global__ void __launch_bounds__(128, MINB) batch_kernel(const __grid_constant_
   constexpr int G = T::kRawRegs == 4 ? (CH == 1 && MINB == 4 ? 16 : 8) : 16, GF = CH == 1 && MINB == 4 ? 16 : 8;
   // rows of a scan step in flight per lane: 64 registers, 32 in the smaller builds
   constexpr int kRows = (MINB == 4 ? 16 : 8) / T::kRawRegs, RB = kRows > 8 ? 8 : kRows;
+  // Narrow rows in the smaller builds: each load takes a part of a line, and the warps beside
+  // it are many; with the line kept in L1, 10,000 auto-routed queries over 1M x 128 take
+  // BF16 1,674 -> 1,617 us (96 registers) and 2,317 -> 1,859 (80), FP8 1,824 -> 1,705 and
+  // 2,431 -> 2,103. In the 128-register build BF16 loses 7 % (4,000 pre-filter queries).
+  constexpr bool kL1 = MINB > 4 && T::kRawRegs < 4;
   for (int t = threadIdx.x; t < (int)(sizeof(BatchArgs) / 4); t += blockDim.x)
     reinterpret_cast<uint32_t*>(smem_raw)[t] = reinterpret_cast<const uint32_t*>(&a)[t];
   __syncthreads();
@@ -794,7 +805,7 @@ __global__ void __launch_bounds__(128, MINB) batch_kernel(const __grid_constant_
       const int64_t at = idx < nL ? a.cap_nq + idx : idx < nLB ? 2 * a.cap_nq + (idx - nL) : 2 * a.cap_nq - 1 - (idx - nLB);
       graph_query<T, CH, G, GF, S1>(a, w, a.queues[at], hy);
     } else if (!a.skip_scan && idx - nG < __ldg(a.counters + CNT_ITEMS)) {
-      scan_item<T, CH, RB, GF>(w.off, idx - nG);
+      scan_item<T, CH, RB, GF, kL1>(w.off, idx - nG);
     } else {
       break;
     }

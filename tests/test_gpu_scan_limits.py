@@ -29,3 +29,41 @@ def test_small_tensor_core_batch_after_a_large_one(nq, c2_small_index):
         np.testing.assert_array_equal(r["ids"], ids[rows])
         np.testing.assert_array_equal(r["count"], cnt[rows])
     ix.close()
+
+
+@pytest.mark.parametrize("k,mult", [(1, 1), (33, 4), (256, 16)])
+def test_pre_filter_lists_without_walk_buffers(k, mult, c2_small_index):
+    """A forced pre-filter batch gets shared memory for its lists alone, whatever the walks'
+    parameters: up to 4,096 candidates re-ranked, the smallest and a large beam."""
+    import oracle
+    import paper_2412_02448_gb300 as U
+    w, path = c2_small_index
+    rows = np.arange(60)
+    ids, _, cnt = oracle.exact_knn(w.vectors, w.attrs, w.queries[rows], w.lo[rows], w.hi[rows], k)
+    ix = U.Index(path, device=0)
+    for dtype in (U.FP32, U.BF16):  # coordinates up to 255 are exact in both
+        for kw in (dict(visited_cap=64, cand_cap=32, ef=1), dict(visited_cap=8192, cand_cap=2048, ef=300)):
+            r = _run(ix, w, rows, k, dtype=dtype, rerank_mult=mult, warps_per_block=2, **kw)
+            np.testing.assert_array_equal(r["ids"], ids)
+            np.testing.assert_array_equal(r["count"], cnt)
+    ix.close()
+
+
+@pytest.mark.parametrize("dtype", [0, 1, 2])
+def test_routed_scans_in_every_build(dtype, c2_small_index):
+    """Pre-filter items of a routed batch in the builds of 128, 96 and 80 registers (which load
+    narrow rows in two ways), next to walks: the same rows."""
+    import paper_2412_02448_gb300 as U
+    import torch
+    w, path = c2_small_index
+    ix = U.Index(path, device=0)
+    out = []
+    for regs in (128, 80, 64):
+        p = U.Params.defaults(dtype=dtype, reg_budget=regs, tau_a=w.n // 10, tau_b=w.n // 2, rerank_mult=2)
+        r = ix.search(w.queries, w.lo, w.hi, 10, strategy="auto", params=p)
+        torch.cuda.synchronize()
+        out.append({n: v.cpu().numpy() for n, v in r.items()})
+    for r in out[1:]:
+        for n in ("ids", "dist", "count"):
+            np.testing.assert_array_equal(r[n], out[0][n])
+    ix.close()
