@@ -279,7 +279,7 @@ __device__ __forceinline__ int select_s1(const BatchArgs& a, const WarpMem& w, i
   for (int b0 = 0; b0 < tot; b0 += 32) {
     const int cid = next;
     next = neighbour(b0 + 32 + lane);
-    const float dv = batch_dist<T, CH, G, CH == 1 && T::kRawRegs == 1>(w.xo(), cid, a.vt, a.row_bytes, a.scale, a.dp4, scratch);
+    const float dv = batch_dist<T, CH, G>(w.xo(), cid, a.vt, a.row_bytes, a.scale, a.dp4, scratch);
     ns = topk_offer(selk, ns, a.m < 64 ? a.m : 64, cid >= 0 ? make_key(dv, cid) : kKeyMax, w.SK(), a.repeats != 0);
   }
   for (int t = lane; t < ns; t += 32) sts32(w.nadj(0) + 4 * t, key_id(lds64(selk + 8 * t)));

@@ -166,48 +166,7 @@ __device__ __forceinline__ float hex_dist(saddr qs, saddr clist, int n, const un
   return __shfl_sync(kFull, v[0], ((lane & 1) * 16 + (lane >> 1) * (16 / R)) & 31);
 }
 
-// The same with a whole warp per row (lane L holds chunk L, rows of at most 32 chunks):
-// one load instruction takes one line of a 128-byte FP8 row instead of a quarter of four.
-// The same tree, its first levels as shuffles too. For S1 over FP8 rows, whose expansions
-// take the distances of up to 256 neighbours to their owner and are bound by the loads'
-// line lookups (3,696 queries on GB300: 2,028 -> 1,964 us). Walks over FP8 rows are slower
-// with it (log-uniform batch of 5,001: 1,258 -> 1,561 us).
-template <class T, int G>
-__device__ __forceinline__ float line_dist(saddr qs, saddr clist, int n, const unsigned char* rows, int row_bytes,
-                                           const float* scale, int dp4) {
-  const int lane = lane_id();
-  const int c = lane < dp4 ? lane : dp4 - 1;
-  Held<T> x[G];
-  float v[G];
-#pragma unroll
-  for (int u = 0; u < G; ++u) {
-    const int id = lds32(clist + 4 * (u < n ? u : n - 1)) & kIdMask;
-    x[u] = T::load_raw(rows + (int64_t)id * row_bytes, c);
-    v[u] = T::kScaled ? __ldg(scale + id) : 1.f;
-  }
-  const float4 q = lds_f4(qs + 16 * c);
-#pragma unroll
-  for (int u = 0; u < G; ++u) {
-    const float s = sum_sq<T>(q, T::decode(x[u]), v[u], 0.f);
-    v[u] = lane < dp4 ? s : 0.f;
-  }
-  int off = 16;
-#pragma unroll
-  for (int cnt = G; cnt > 1; cnt >>= 1, off >>= 1) {
-    const bool up = (lane & off) != 0;
-#pragma unroll
-    for (int i = 0; i < cnt / 2; ++i) {
-      const float send = up ? v[i] : v[i + cnt / 2];
-      const float keep = up ? v[i + cnt / 2] : v[i];
-      v[i] = keep + __shfl_xor_sync(kFull, send, off);
-    }
-  }
-#pragma unroll
-  for (; off >= 1; off >>= 1) v[0] += __shfl_xor_sync(kFull, v[0], off);
-  return __shfl_sync(kFull, v[0], (lane * (32 / G)) & 31);  // candidate u sits in lane u * (32 / G)
-}
-
-template <class T, int CH, int G, bool kLine = false>
+template <class T, int CH, int G>
 __device__ __forceinline__ float group_dist(saddr qs, saddr clist, int nv, const unsigned char* rows, int row_bytes,
                                             const float* scale, int dp4) {
   const int lane = lane_id();
@@ -225,9 +184,7 @@ __device__ __forceinline__ float group_dist(saddr qs, saddr clist, int nv, const
   for (int base = 0; base < nv; base += kStep) {
     const int n = nv - base;
     float v;
-    if constexpr (kLine) {
-      v = line_dist<T, G>(qs, clist + 4 * base, n, rows, row_bytes, scale, dp4);
-    } else if constexpr (CH >= 4) {
+    if constexpr (CH >= 4) {
       v = hex_dist<T, CH, kStep / 2>(qs, clist + 4 * base, n, rows, row_bytes, scale, dp4);
     } else {
       // half a group where that is enough: half the instructions
@@ -242,7 +199,7 @@ __device__ __forceinline__ float group_dist(saddr qs, saddr clist, int nv, const
 
 // The same for candidates held by the lanes (cid >= 0): each such lane gets its own
 // candidate's distance. clist is 32 ints of per-warp shared scratch.
-template <class T, int CH, int G, bool kLine = false>
+template <class T, int CH, int G>
 __device__ __forceinline__ float batch_dist(saddr qs, int cid, const unsigned char* rows, int row_bytes,
                                             const float* scale, int dp4, saddr clist) {
   const unsigned vm = __ballot_sync(kFull, cid >= 0);
@@ -250,7 +207,7 @@ __device__ __forceinline__ float batch_dist(saddr qs, int cid, const unsigned ch
   __syncwarp();
   if (cid >= 0) sts32(clist + 4 * my, cid);
   __syncwarp();
-  const float d = group_dist<T, CH, G, kLine>(qs, clist, __popc(vm), rows, row_bytes, scale, dp4);
+  const float d = group_dist<T, CH, G>(qs, clist, __popc(vm), rows, row_bytes, scale, dp4);
   return __shfl_sync(kFull, d, my & 31);
 }
 
