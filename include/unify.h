@@ -100,7 +100,8 @@ typedef struct {
   int reg_budget;      /* build of the search kernel for rows of up to 128 elements: 128 (128 registers
                           per thread, 16 warps per SM), 80 (96 registers, 20 warps) or 64 (80
                           registers, 24 warps; the smaller builds hold fewer rows in flight per
-                          warp); default 128. More resident warps hide more memory latency when
+                          warp); default 128. Selection S1 always runs the 128 build (the
+                          others are slower there). More resident warps hide more memory latency when
                           shared memory (cand_cap, visited_cap, ef) also fits. */
   int tc_scan;         /* 1: Strategy A queries are scanned on the tensor cores (tcgen05 MMA
                           over TMA-staged row tiles shared by 128 queries; bf16 operands for

@@ -772,13 +772,17 @@ __device__ __noinline__ void scan_item(uint32_t off, int it) {
 }
 
 // MINB: minimum resident CTAs of 128 threads per SM the register allocation must
-// allow (4 -> 128 registers, 6 -> 80, 8 -> 64). A group of distances holds up to 64
+// allow (4 -> 128 registers, 5 -> 96, 6 -> 80). A group of distances holds up to 64
 // registers of row chunks in flight (32 in the smaller builds), the scan as well.
 template <class T, int CH, int MINB, bool S1>
 __global__ void __launch_bounds__(128, MINB) batch_kernel(const __grid_constant__ BatchArgs a) {
   // rows per distance group: 64 registers of row chunks in flight, 32 in the smaller builds
-  // and for rows of more than 128 elements (there a block of each row at a time)
-  constexpr int G = T::kRawRegs == 4 ? (CH == 1 && MINB == 4 ? 16 : 8) : 16, GF = CH == 1 && MINB == 4 ? 16 : 8;
+  // and for rows of more than 128 elements (there a block of each row at a time). Selection
+  // S1 over FP8 rows takes 8: its expansions decode up to 256 neighbours next to the query's
+  // (GB300, 3,696 queries over 1M x 128: 1,877 -> 1,625 us; 2,000 hybrid ones 2,327 -> 2,209;
+  // 5,000 log-uniform ones over 200K x 96 3,266 -> 3,378).
+  constexpr int G = T::kRawRegs == 4 ? (CH == 1 && MINB == 4 ? 16 : 8) : S1 && T::kRawRegs == 1 ? 8 : 16,
+                GF = CH == 1 && MINB == 4 ? 16 : 8;
   // rows of a scan step in flight per lane: 64 registers, 32 in the smaller builds
   constexpr int kRows = (MINB == 4 ? 16 : 8) / T::kRawRegs, RB = kRows > 8 ? 8 : kRows;
   // Narrow rows in the smaller builds: each load takes a part of a line, and the warps beside
@@ -828,7 +832,9 @@ static cudaError_t launch_t(const BatchArgs& a, int wpb, int num_sms, cudaStream
 }
 
 // The build for a row width (CH * 32 chunks of 4 elements hold a row), a register budget
-// (rows of up to 128 elements) and the hybrid selection.
+// (rows of up to 128 elements) and the hybrid selection. S1 has the 128-register build alone:
+// its second query row and key list spill in smaller ones (GB300, 3,696 queries over 1M x
+// 128, 128 / 96 / 80 registers: float32 1,805 / 1,935 / 2,065 us, BF16 1,815 / 2,050 / 2,250).
 template <class T>
 static cudaError_t launch_dt(const BatchArgs& a, int wpb, int regs, int num_sms, cudaStream_t st) {
   const int ch = (a.dp4 + 31) / 32;
