@@ -11,11 +11,11 @@ namespace unify {
 // never below 64 rows, nor below 4 rows per key kept (each item sorts its own list of the
 // kept keys, which the query's last item merges). In a routed batch the graph walks hold most
 // warps for longer than an item takes, and finer items only take issue slots from them (2 %
-// slower at 1,003 queries with 64 KB): there a batch counts sixteenfold, up to 512 KB, beyond
-// which the items after the walks are too few for an even end: 5,000 log-uniform queries
-// over 1M x 128 at the tuned parameters 2,091 us with 4 MB, 1,863 with 1 MB, 1,878 with 512
-// KB, 2,042 with 64 KB; 10,000 queries of five widths 2,065, 1,970, 1,974 and 2,095; 5,000
-// of these 1,119, 1,062, 1,023 and 1,083.
+// slower at 1,003 queries with 64 KB): there a batch counts sixteenfold, up to 1 MB. Above
+// that the items behind the walks are too few for an even end, below it they slow the long
+// walks. With 4 MB / 1 MB / 512 KB / 256 KB, 1M x 128 at the tuned parameters: 5,000
+// log-uniform queries 2,108 / 1,867 / 1,878 / 1,917 us, 10,000 of five widths 2,061 / 1,970 /
+// 1,973 / 2,002; 5,001 log-uniform queries over 200K x 96 FP8 1,281 / 1,276 / 1,299 / 1,305.
 // Measured on GB300 against items of 8,192 rows: 17 queries over 15,000 rows of 512 B
 // each 585 -> 50 us; 301 queries over 4,200 rows of 3,840 B 4,900 -> 609 us.
 int scan_item_rows(const DeviceIndex& ix, const Params& p, int64_t nq, int strategy) {
@@ -23,7 +23,7 @@ int scan_item_rows(const DeviceIndex& ix, const Params& p, int64_t nq, int strat
   const int64_t slots = 16ll * ix.num_sms;
   int64_t bytes = (1ll << 20) * (strategy == UNIFY_AUTO ? 16 : 1) * nq / slots;
   if (bytes < (64 << 10)) bytes = 64 << 10;
-  const int64_t most = strategy == UNIFY_AUTO ? 512 << 10 : 4 << 20;
+  const int64_t most = strategy == UNIFY_AUTO ? 1 << 20 : 4 << 20;
   if (bytes > most) bytes = most;
   const int64_t kept = rerank_count(p) > p.k ? rerank_count(p) : p.k;
   int64_t rows = bytes / row_bytes;
