@@ -426,8 +426,8 @@ def run(args):
     def algorithmic_bytes(params, counters, k):
         """Bytes the search kernel must move per launch, by strategy: a scanned row
         (its storage bytes plus the 4-byte id) per in-range row for A; per distance
-        evaluation one row, and per expansion the adjacency slots read (S' chunks of
-        ceil(m / S') slots for C; M slots plus the bitmap words for B); plus the FP32
+        evaluation one row, and per expansion the neighbour ids read (S' chunks of
+        ceil(m / S') slots for C; the marked ids, at most M of a row, for B); plus the FP32
         re-rank rows of the BF16/FP8 paths."""
         isA, isB, isC = routing(params)
         row = {U.FP32: 4 * d, U.BF16: 2 * d, U.FP8E4M3: d + 4}[params.dtype]
@@ -436,8 +436,7 @@ def run(args):
         return {
             "scan": float(((pb - pa) * (row + 4))[isA].sum() + rr * isA.sum()),
             "hybrid": float((counters[isC, 0] * row + counters[isC, 1] * Sp[isC] * per[isC] * 4).sum() + rr * isC.sum()),
-            "post": float((counters[isB, 0] * row + counters[isB, 1] * (ix.M + (ix.S * ix.M + 31) // 32) * 4).sum()
-                          + rr * isB.sum()),
+            "post": float((counters[isB, 0] * row + counters[isB, 1] * ix.M * 4).sum() + rr * isB.sum()),
         }
 
     def scored(ids, k):

@@ -31,7 +31,7 @@
 //
 // Bounds (checked against the buffers of each launch): warps cover
 // count * S pairs (a warp-uniform early return past the end); neighbour slots are
-// read for lane < cnt <= M <= 32; E holds at most ecap >= efc keys; kept at most
+// read for lane < M <= 32, and those past a chunk's count hold -1; E holds at most ecap >= efc keys; kept at most
 // M <= 32 keys; output rows are row0[v] + l - row0[first] < rows of the batch. The
 // reverse-edge warps hold at most M + 1 <= 33 candidate keys; group chunks, group
 // bounds and sources are validated on the host before upload.
@@ -70,7 +70,6 @@ struct BuildArgs {
   const int32_t* level;
   const int64_t* row0;
   const int32_t* adj;  // nrows x S x M
-  const uint8_t* cnt;  // nrows x S
   int S, M, efc, ecap;
   int32_t entry_seg[kBuildMaxS], top_seg[kBuildMaxS];
   int64_t first, count, row_first;
@@ -569,7 +568,6 @@ int propose(BuildCtx* c, const unify_build_view_t* v, int32_t* out_ids, float* o
   a.level = c->level;
   a.row0 = c->row0;
   a.adj = c->adj;
-  a.cnt = c->cnt;
   a.S = c->S;
   a.M = c->M;
   a.efc = v->efc;

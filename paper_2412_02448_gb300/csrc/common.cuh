@@ -155,10 +155,11 @@ __device__ __forceinline__ float oct_transpose_reduce(float (&v)[V]) {
 //
 // Raw is a chunk as loaded (16, 8 or 4 bytes: 4, 2 or 1 registers); decode() turns it
 // into four floats, at use.
+//
 // Read-only loads that leave no line in L1 (kL1: that do): a row is read once by its warp,
-// and the L1 beside a full shared memory is small. Volatile: all loads of a group stay together in
-// front of the arithmetic. Otherwise the compiler moves each into the branch that uses
-// its chunk, and a group costs four memory latencies instead of one.
+// and the L1 beside a full shared memory is small. Volatile: all loads of a group stay
+// together in front of the arithmetic. Otherwise the compiler moves each into the branch
+// that uses its chunk, and a group costs four memory latencies instead of one.
 template <bool kL1>
 __device__ __forceinline__ float4 load_stream16(const void* p) {
   float4 v;

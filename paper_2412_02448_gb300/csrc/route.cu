@@ -63,7 +63,6 @@ struct RouteArgs {
   int64_t cap_nq;
   int2* items;
   int32_t* counters;
-  int32_t* out_count;     // may be null (set 0 for empty pre-filter queries handled here)
   int32_t* out_counters;  // may be null
   // tensor-core scan: its tables to clear (slots to -1, spans to 0); null without it
   int32_t* tc_slotpos;
@@ -114,8 +113,8 @@ __global__ void __launch_bounds__(32 * kRouteWarps) route_kernel(RouteArgs a, co
       // post-filter walk (an expansion of theirs costs about 1.5 of one) go before those,
       // the others after. Measured on GB300, 10,000 auto-routed queries over 1M x 128 (4,000
       // short hybrid walks, 2,000 post-filter walks; all hybrid walks first before):
-      // float32 1,259 -> 1,096 us, bfloat16 1,182 -> 1,010 us. Post-filter walks before every hybrid one lost 8 % on a batch with ranges
-      // that fill a tenth of their segments.
+      // float32 1,259 -> 1,096 us, bfloat16 1,182 -> 1,010 us. Post-filter walks before every
+      // hybrid one lost 8 % on a batch with ranges that fill a tenth of their segments.
       const unsigned rows = hit ? (unsigned)(__ldg(seg_start + lane + 1) - __ldg(seg_start + lane)) : 0u;
       const int64_t met = __reduce_add_sync(kFull, rows);
       shrt = 3 * (int64_t)a.ef_h * met <= 2 * (int64_t)a.ef_p * Y;
@@ -220,7 +219,6 @@ cudaError_t launch_route(const DeviceIndex& ix, const Scratch& sc, const int64_t
   a.cap_nq = sc.cap_nq;
   a.items = sc.items;
   a.counters = sc.counters;
-  a.out_count = outs ? outs->count : nullptr;
   a.out_counters = outs ? outs->counters : nullptr;
   a.tc_slotpos = tc ? sc.tc_slotpos : nullptr;
   a.tc_slots = sc.tc_slots;

@@ -5,9 +5,9 @@
 // each pre-filter query into scan items. One warp takes one work unit at a time
 // from a single device counter, in the order: long hybrid walks, post-filter walks,
 // short hybrid walks (route.cu tells them apart), scan items. The long graph searches
-// start first and the short scan items fill the tail, so the batch has one tail instead of one per strategy. A pre-filter
-// query split into several items is merged by the warp that completes its last
-// item (release/acquire through a per-query counter).
+// start first and the short scan items fill the tail, so the batch has one tail instead of
+// one per strategy. A pre-filter query split into several items is merged by the warp that
+// completes its last item (release/acquire through a per-query counter).
 //
 // Graph search (Algorithm 2's scheme; Algorithm 1 for B over bitmap-marked
 // slots; Algorithm 7 for C over the first ceil(m/S') slots of each intersected
@@ -43,10 +43,12 @@
 //   - a group's row loads are all in flight together (group_dist);
 //   - the insertion needs no sort: ranks by counting, and every position of a sorted
 //     array finds its source by a ballot (sorted_insert);
-//   - nothing is spilled in the loop: with shared memory full, L1 is small and swept by
-//     the row gathers, and a reload of a spilled register comes from L2. State that an
-//     expansion seldom needs lives in shared memory, scan and re-rank run out of line,
-//     hybrid and post walks share one body, and addresses are recomputed (WarpMem).
+//   - few registers are spilled: with shared memory full, L1 is small and swept by the row
+//     gathers, and a reload of a spilled register comes from L2. State that an expansion
+//     seldom needs lives in shared memory, scan and re-rank run out of line, hybrid and post
+//     walks share one body, and addresses are recomputed (WarpMem). The builds for rows of up
+//     to 128 elements still report 16 to 72 bytes of spill stores with 128 and 96 registers and
+//     96 to 142 with 80; how many of them lie inside the loop was not established.
 // Measured on GB300 against lanes-per-row of 32, a bitonic sort, a merge by binary
 // searches and 32 to 136 bytes of spills per thread: one query, 120 expansions 399 -> 276
 // us; 10,000 auto-routed queries over 1M x 128 (graph walks and the tensor-core scan
@@ -56,8 +58,9 @@
 // Scan (Strategy A): rows [pa, pb) of the attribute-ordered vectors; a warp
 // computes 32 rows per step, eight lanes per row (4 shuffles per 16 rows instead of 16,
 // all loads of a batch in flight); keys beating the current k-th are inserted into a
-// sorted top-k. Bound by HBM once a batch fills the device: 301 queries over 4,150 rows of
-// 3,840 B each run at 4.9 TB/s of gathered rows (985 us).
+// sorted top-k. Bound by the latency of a step's loads and by L2 and HBM: 301 queries over
+// 4,150 rows of 3,840 B each gather 8 TB/s (609 us), 4,000 queries over 1M x 128 float32 8.4
+// TB/s (1,347 us).
 //
 // Bounds (checked by reading, against the buffers the launch receives):
 // E[< cand_cap], ann[< ann_cap], vis[< 2^vis_log2], clist[< 32], SK[< 32], nadj and
@@ -324,10 +327,10 @@ __device__ __forceinline__ void insert_batch(const BatchArgs& a, const WarpMem& 
 }
 
 // One layer (cold()->l; base: layer 0) of Algorithm 1 (post) or Algorithm 7 (hybrid, hy;
-// S1: with that selection) over cold()->slots slots per expansion. Returns |ann|; the ann array is w.ann for hybrid. For
-// post every candidate push is also an ann push, so cand is a subset of ann and one
-// sorted buffer of capacity efl holds both: the result is then in w.ann as well (the
-// buffer is w.ann itself, its flags set).
+// S1: with that selection) over cold()->slots slots per expansion. Returns |ann|; the ann
+// array is w.ann for hybrid. For post every candidate push is also an ann push, so cand is
+// a subset of ann and one sorted buffer of capacity efl holds both: the result is then in
+// w.ann as well (the buffer is w.ann itself, its flags set).
 template <class T, int CH, int G, bool S1>
 __device__ __forceinline__ int search_layer(const BatchArgs& a, WarpMem w, bool hy, bool base, int efl, uint64_t ep_key,
                                             bool ep_in) {
@@ -833,7 +836,7 @@ static cudaError_t launch_t(const BatchArgs& a, int wpb, int num_sms, cudaStream
 
 // The build for a row width (CH * 32 chunks of 4 elements hold a row), a register budget
 // (rows of up to 128 elements) and the hybrid selection. S1 has the 128-register build alone:
-// its second query row and key list spill in smaller ones (GB300, 3,696 queries over 1M x
+// the smaller ones spill more (GB300, 3,696 queries over 1M x
 // 128, 128 / 96 / 80 registers: float32 1,805 / 1,935 / 2,065 us, BF16 1,815 / 2,050 / 2,250).
 template <class T>
 static cudaError_t launch_dt(const BatchArgs& a, int wpb, int regs, int num_sms, cudaStream_t st) {
