@@ -102,7 +102,8 @@ typedef struct {
                           registers, 24 warps; the smaller builds hold fewer rows in flight per
                           warp); default 128. Selection S1 always runs the 128 build (the
                           others are slower there). More resident warps hide more memory
-                          latency when shared memory (cand_cap, visited_cap, ef) also fits. */
+                          latency; where shared memory (cand_cap, visited_cap, ef) admits no
+                          more of them, the larger build runs. */
   int tc_scan;         /* 1: Strategy A queries are scanned on the tensor cores (tcgen05 MMA
                           over TMA-staged row tiles shared by 128 queries; bf16 operands for
                           UNIFY_BF16 storage, tf32 for UNIFY_FP32, E4M3 for UNIFY_FP8E4M3; the

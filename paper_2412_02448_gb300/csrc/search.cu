@@ -49,6 +49,18 @@ int batch_smem_per_warp(const Params& p) {
   return (p.cand_cap * 8 + ann * 8 + (4 << p.vis_log2) + ((big + 15) & ~15) + 768 + 15) & ~15;
 }
 
+// The build that reg_budget asks for, or the next larger one where shared memory admits no
+// more warps per SM than that holds (16 at 128 registers, 20 at 96): a smaller build then
+// only has fewer rows in flight per warp. An SM has 228 KB, 1 KB of it lost per CTA.
+// Measured on GB300 with the default buffers (12 warps fit), reg_budget 64 in the
+// 80-register build / in the 128-register build: 6,000 hybrid queries over 1M x 128 float32
+// 3,871 / 2,956 us, 6,000 post-filter ones 1,604 / 1,266, 2,111 short ranges 505 / 408.
+static int usable_reg_budget(int asked, int cta_bytes, int wpb) {
+  const int warps = 228 * 1024 / (cta_bytes + 1024) * wpb;
+  if (warps <= 16) return 128;
+  return warps <= 20 && asked == 64 ? 80 : asked;
+}
+
 cudaError_t launch_batch(const DeviceIndex& ix, const Scratch& sc, const float* q, const Params& p,
                          const Outputs& o, cudaStream_t st, bool skip_scan, const Conj* cj, bool scan_only) {
   BatchArgs a;
@@ -110,6 +122,7 @@ cudaError_t launch_batch(const DeviceIndex& ix, const Scratch& sc, const float* 
   a.ann_cap = batch_ann_cap(p);
   a.vis_log2 = p.vis_log2;
   a.max_exp = p.max_exp;
+  a.scan_only = scan_only ? 1 : 0;
   if (scan_only) {
     // Nothing walks: no visited filter, the lists alone. With the default parameters 16 warps
     // per SM instead of the 12 that fit beside the walks' buffers (the 128-register build):
@@ -123,9 +136,10 @@ cudaError_t launch_batch(const DeviceIndex& ix, const Scratch& sc, const float* 
   const int fit = (227 * 1024 - kArgsBytes) / a.warp_bytes;
   const int wpb = p.warps_per_block < fit ? p.warps_per_block : fit;
   if (wpb < 1) return cudaErrorInvalidConfiguration;
-  if (p.dtype == UNIFY_BF16) return launch_batch_bf16(a, wpb, p.reg_budget, ix.num_sms, st);
-  if (p.dtype == UNIFY_FP8E4M3) return launch_batch_fp8(a, wpb, p.reg_budget, ix.num_sms, st);
-  return launch_batch_f32(a, wpb, p.reg_budget, ix.num_sms, st);
+  const int regs = usable_reg_budget(p.reg_budget, kArgsBytes + wpb * a.warp_bytes, wpb);
+  if (p.dtype == UNIFY_BF16) return launch_batch_bf16(a, wpb, regs, ix.num_sms, st);
+  if (p.dtype == UNIFY_FP8E4M3) return launch_batch_fp8(a, wpb, regs, ix.num_sms, st);
+  return launch_batch_f32(a, wpb, regs, ix.num_sms, st);
 }
 
 }  // namespace unify

@@ -114,6 +114,7 @@ struct BatchArgs {
   int repeats;  // a row of the file may name a neighbour more than once
   int s1;  // hybrid selection S1 (the m neighbours nearest to the expanded object) instead of S2
   int warp_bytes, off_q, off_E, off_ann;
+  int scan_only;  // every query is a pre-filter query: no walks' buffers, a large L1
   int skip_scan;  // the pre-filter queries were searched by the tensor-core scan
   Outputs o;
 };
@@ -665,7 +666,7 @@ static __device__ __noinline__ int merge_lists(saddr off, const uint64_t* lists,
   return nt;
 }
 
-template <class T, int CH, int RB, int GF, bool kL1>
+template <class T, int CH, int RB, int GF, bool kL1, bool kEarly>
 __device__ __noinline__ void scan_item(uint32_t off, int it) {
   const BatchArgs& a = shared_args();
   const WarpMem w{off, a};
@@ -696,6 +697,9 @@ __device__ __noinline__ void scan_item(uint32_t off, int it) {
   int nt = 0;
 #pragma unroll 1
   for (int base = r0; base < r1; base += 32) {
+    // the ids of short rows on their way with them (4,000 queries over 1M x 128 BF16 954 ->
+    // 907 us; long rows lose 4 %, the smaller builds up to 3 %)
+    const int32_t id0 = kEarly ? __ldg(sorted_ids + min(base + 4 * j + g, r1 - 1)) : 0;
     float part[8];
 #pragma unroll
     for (int h = 0; h < 8; h += RB) {
@@ -737,7 +741,7 @@ __device__ __noinline__ void scan_item(uint32_t off, int it) {
     const int row = base + 4 * j + g;
     uint64_t key = kKeyMax;
     if (row < r1) {
-      const int32_t id = __ldg(sorted_ids + row);
+      const int32_t id = kEarly ? id0 : __ldg(sorted_ids + row);
       if (conj_ok(a, id, l2, h2)) key = make_key(dist, id);
     }
     nt = topk_offer(topk, nt, kk, key, w.SK());
@@ -788,11 +792,15 @@ __global__ void __launch_bounds__(128, MINB) batch_kernel(const __grid_constant_
                 GF = CH == 1 && MINB == 4 ? 16 : 8;
   // rows of a scan step in flight per lane: 64 registers, 32 in the smaller builds
   constexpr int kRows = (MINB == 4 ? 16 : 8) / T::kRawRegs, RB = kRows > 8 ? 8 : kRows;
-  // Narrow rows in the smaller builds: each load takes a part of a line, and the warps beside
-  // it are many; with the line kept in L1, 10,000 auto-routed queries over 1M x 128 take
-  // BF16 1,674 -> 1,617 us (96 registers) and 2,317 -> 1,859 (80), FP8 1,824 -> 1,705 and
-  // 2,431 -> 2,103. In the 128-register build BF16 loses 7 % (4,000 pre-filter queries).
-  constexpr bool kL1 = MINB > 4 && T::kRawRegs < 4;
+  // Scans keep the lines of short narrow rows in L1, of which each load takes a part, and
+  // beside the walks' buffers, which leave L1 little room for loads that bypass it, also those
+  // of float32 rows where no walk shares L1 (decided below). GB300, without / with: 10,000
+  // auto-routed queries over 1M x 128 BF16 1,627 / 1,581 us (96 registers 1,674 / 1,603, 80
+  // registers 2,317 / 1,858), 4,000 short ranges BF16 1,211 / 1,133, 4,000 over 200K x 96 BF16
+  // 321 / 296, float32 331 / 277; against it: 1,003 float32 queries with walks 1,900 / 1,938,
+  // 4,000 forced pre-filter ones BF16 907 / 932 (a second copy of the scan for these cost the
+  // BF16 walks 1.5 %).
+  constexpr bool kL1 = CH == 1 && T::kRawRegs < 4, kEarly = CH == 1 && MINB == 4;
   for (int t = threadIdx.x; t < (int)(sizeof(BatchArgs) / 4); t += blockDim.x)
     reinterpret_cast<uint32_t*>(smem_raw)[t] = reinterpret_cast<const uint32_t*>(&a)[t];
   __syncthreads();
@@ -812,7 +820,8 @@ __global__ void __launch_bounds__(128, MINB) batch_kernel(const __grid_constant_
       const int64_t at = idx < nL ? a.cap_nq + idx : idx < nLB ? 2 * a.cap_nq + (idx - nL) : 2 * a.cap_nq - 1 - (idx - nLB);
       graph_query<T, CH, G, GF, S1>(a, w, a.queues[at], hy);
     } else if (!a.skip_scan && idx - nG < __ldg(a.counters + CNT_ITEMS)) {
-      scan_item<T, CH, RB, GF, kL1>(w.off, idx - nG);
+      if (CH == 1 && MINB == 4 && nG == 0 && !a.scan_only) scan_item<T, CH, RB, GF, true, kEarly>(w.off, idx - nG);
+      else scan_item<T, CH, RB, GF, kL1, kEarly>(w.off, idx - nG);
     } else {
       break;
     }
